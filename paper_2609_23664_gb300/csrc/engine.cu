@@ -58,12 +58,36 @@ void launch_copy(const void *src, void *dst, size_t bytes, void *stream) {
 // ---------------------------------------------------------------------------
 // device-side tables of a set of statevector programs
 // ---------------------------------------------------------------------------
+// Writes {1, t; -t, 1} as diag(1, a1) {1, T0; T1, 1} diag(1, 1 / a1) with T0
+// and T1 exact in FP32, and returns a1.  That needs T0 T1 = -t^2: with
+// s t in [2^22, 2^23] for a power of two s, A an integer just above s t and
+// k the integer nearest sqrt(A^2 - (s t)^2), (A + k)(A - k) differs from
+// (s t)^2 by at most k < 2^14, that is 2^-31 of it; the best of eight A is
+// taken (2^-34 typically), a1 = (A + k) / (s t) = 1 + O(2^-10).
+static double exact_rotation(double t, float T[2]) {
+  T[0] = T[1] = 0.f;
+  if (!(std::fabs(t) > 1e-30)) return 1.0;
+  int ex;
+  std::frexp(std::fabs(t), &ex);
+  const double st = std::ldexp(std::fabs(t), 23 - ex), tau = st * st;
+  double A = 0, k = 0, best = 1e300;
+  const double a0 = std::ceil(st);
+  for (int i = 0; i < 8; i++) {
+    const double a = a0 + i, kk = std::nearbyint(std::sqrt(a * a - tau)), r = std::fabs(a * a - kk * kk - tau);
+    if (r < best) { best = r; A = a; k = kk; }
+  }
+  const double unit = std::ldexp(t < 0 ? -1.0 : 1.0, ex - 23);
+  T[0] = (float)((A + k) * unit);
+  T[1] = (float)(-(A - k) * unit);
+  return (A + k) / st;
+}
+
 struct SvTableBuilder {
   std::vector<SvPassDesc> passes;
   std::vector<SvStageDesc> stages;
   std::vector<SvOpDesc<float>> ops32;
   std::vector<float> ops32lo;  // m[t] - (float)m[t] per FP32 op (compensated passes)
-  std::vector<float> ph;       // phase products of full rotation-and-phase stages (FP32)
+  std::vector<float> ph;       // blocks of the compensated rotation stages (see SvStageDesc::ph_block)
   std::vector<SvOpDesc<double>> ops64;
   bool fp64;
   explicit SvTableBuilder(bool f) : fp64(f) {}
@@ -224,28 +248,50 @@ struct SvTableBuilder {
             }
         }
         sd.rp_mask = rp_stage ? rp_mask : 0u;
-        // a stage of four-position groups with a rotation-and-phase op on
-        // every position is D R3 R2 R1 R0 with D the product of the ops'
-        // |1>-phases (each diagonal on its own position, so it commutes
-        // with the other positions' rotations): amplitude e of the group
-        // takes the product of the phases of its set positions, computed
-        // here in FP64 and stored as double-float pairs
+        // a compensated stage of rotations: each real orthogonal 2x2
+        // {r00, r01; r10, r11} is diag(r00, r11) {1, r01/r00; r10/r11, 1};
+        // where |r01| is the larger entry the columns are exchanged first
+        // (the group is read with that position's halves exchanged), so the
+        // off-diagonal quotients stay within 1.  The diagonals commute with
+        // the other positions' rotations: amplitude e takes their product,
+        // with the |1>-phases of its set positions, computed here in FP64
+        // and stored as FP32 pairs
         sd.ph_block = 0xFFFFFFFFu;
-        if ((hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0) && (fp64 || pr.g != 4 || !rp_stage || rp_mask != 0xFu))
-          fail(QW_ERR_STATE, "internal: a global phase on a stage without a phase table");
-        if (!fp64 && pr.g == 4 && rp_stage && rp_mask == 0xFu) {
-          const bool gfold = hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0;
-          sd.ph_block = (uint32_t)(ph.size() / 64) | (gfold ? 0x80000000u : 0u);
+        const bool gfold = hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0;
+        if (gfold && (fp64 || pr.g != 4 || !rp_stage)) fail(QW_ERR_STATE, "internal: a global phase on a stage without a table");
+        if (!fp64 && pr.g == 4 && rp_stage) {
+          sd.ph_block = (uint32_t)(ph.size() / SV_PH_BLOCK);
+          float t[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+          double gin[4] = {1, 1, 1, 1};  // input factor of the position's |1> half
+          std::complex<double> d[4][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}};
+          for (const HostOp &o : sops) {
+            double r00 = o.m[0], r01 = o.m[1], r10 = o.m[2], r11 = o.m[3];
+            if (std::fabs(r01) > std::fabs(r00)) {
+              std::swap(r00, r01);
+              std::swap(r10, r11);
+              sd.ld_xor ^= sd.roff[o.a];
+            }
+            const double a1 = exact_rotation(r01 / r00, t[o.a]);
+            gin[o.a] = 1.0 / a1;
+            d[o.a][0] = r00;
+            d[o.a][1] = r11 * a1 * std::complex<double>(o.m[4], o.m[5]);
+          }
+          for (uint32_t e = 0; e < 16; e++) {
+            double f = 1.0;
+            for (uint32_t p4 = 0; p4 < 4; p4++)
+              if ((e >> p4) & 1u) f *= gin[p4];
+            ph.push_back((float)(f - 1.0));
+          }
+          for (int p4 = 0; p4 < 4; p4++) ph.insert(ph.end(), {t[p4][0], t[p4][1]});
           for (uint32_t e = 0; e < 16; e++) {
             std::complex<double> q(hs.gphase[0], hs.gphase[1]);
-            for (const HostOp &o : sops)
-              if ((e >> o.a) & 1u) q *= std::complex<double>(o.m[4], o.m[5]);
-            const float rh = (float)q.real(), ih = (float)q.imag();
-            ph.push_back(rh);
-            ph.push_back((float)(q.real() - (double)rh));
-            ph.push_back(ih);
-            ph.push_back((float)(q.imag() - (double)ih));
+            for (uint32_t p4 = 0; p4 < 4; p4++) q *= d[p4][(e >> p4) & 1u];
+            for (const double v : {q.real(), q.imag()}) {
+              ph.push_back((float)v);
+              ph.push_back((float)(v - (double)(float)v));
+            }
           }
+          sops.clear();  // the stage runs from its block alone
         }
         sd.n_ops = (uint32_t)sops.size();
         sd.op_begin = (uint32_t)(fp64 ? ops64.size() : ops32.size());
@@ -429,33 +475,27 @@ static void *chain_dst_lo(const DeviceState *D, int ar, size_t p, size_t n) {
 // ops under the arithmetic `ar`, per group of A = 2^g amplitudes:
 //   plain: a real rotation output costs 6 (packed multiply + FMA on both
 //   components), a complex product 6, a general 2x2 output 14;
-//   compensated: every two-term output (df_lin2: 2 multiplies, 6 FMAs and
-//   8 adds per component) costs 44, a general 2x2 output two of them plus a
-//   double-float add (104), and every stage renormalizes each amplitude (6).
+//   compensated (sv_df.cuh): a multiply-accumulate on the grid is 4 FMAs
+//   and a subtraction per component (18 for the amplitude's two), so with
+//   the un-biasing of the operand a two-term output costs 40, an
+//   unnormalized rotation output 18, a general 2x2 output 80, and every
+//   stage splits (6, 10 before rotations) and rounds (4) each amplitude.
 static double pass_flops(const HostPass &hp, uint32_t n, uint32_t g, int ar) {
   const bool comp = ar != SV_AR_PLAIN;
   const double groups = std::ldexp(1.0, (int)n - (int)g), A = std::ldexp(1.0, (int)g);
-  const double lin = comp ? 44.0 : 6.0, cm = comp ? 44.0 : 6.0, u1 = comp ? 104.0 : 14.0;
+  const double lin = comp ? 40.0 : 6.0, cm = comp ? 40.0 : 6.0, u1 = comp ? 80.0 : 14.0;
   double f = 0;
   for (const HostStage &st : hp.stages) {
-    double fg = comp ? A * 6.0 : 0.0;
-    // a compensated four-position stage with a rotation (and phase) on
-    // every position: four rotations and one product per amplitude from the
-    // stage's phase table (every amplitude but the first)
-    if (comp && g == 4 && st.ops.size() == 4) {
+    double fg = comp ? A * 10.0 : 0.0;
+    if (comp) {
       uint32_t mask = 0;
-      bool rot = true;
+      bool rot = !st.ops.empty();
       for (const HostOp &o : st.ops) {
         rot = rot && (o.kind == K_RP || o.kind == K_R) && !(mask & (1u << o.a));
         mask |= 1u << o.a;
       }
-      if (rot && mask == 0xFu) {
-        // rounded amplitudes enter a SV_AR_COMP stage with zero remainders:
-        // its first rotation has no remainder products (2 packed FMAs, 8
-        // flops, per output)
-        const double first = (ar == SV_AR_COMP) ? lin - 8.0 : lin;
-        const bool gfold = st.gphase[0] != 1.0 || st.gphase[1] != 0.0;
-        f += (fg + A * first + 3.0 * A * lin + (gfold ? A : A - 1.0) * cm) * groups;
+      if (rot) {  // unnormalized rotations, then one product per amplitude
+        f += (fg + A * (4.0 + 18.0 * (double)st.ops.size() + cm)) * groups;
         continue;
       }
     }

@@ -127,9 +127,8 @@ struct HostStage {
   uint32_t mc = 0;    // and its constant c
   uint32_t ctl_w[SV_MAX_OUT_CTL] = {0, 0, 0, 0};  // per-tile terms of c (pass's ctl_q)
   std::vector<HostOp> ops;
-  // global phase the stage applies to every amplitude (compensated stages
-  // with a rotation on every position carry the program's, in their phase
-  // table)
+  // global phase the stage applies to every amplitude (the first rotation
+  // stage of a compensated program carries the program's, in its table)
   double gphase[2] = {1.0, 0.0};
   HostStage() { for (uint32_t t = 0; t < 32; t++) mcol[t] = 1u << t; }
 };
@@ -193,6 +192,7 @@ struct SvPassDesc {
   // ctl_tb[i] of the tile index is set (ctl_w[i] = 0: unused)
   uint32_t ctl_tb[SV_MAX_OUT_CTL], ctl_w[SV_MAX_OUT_CTL];
 };
+constexpr uint32_t SV_PH_BLOCK = 16 + 4 * 2 + 16 * 4;  // floats of a rotation stage's block
 struct alignas(16) SvStageDesc {
   uint32_t roff[SV_G];           // byte offset of phi(e_pos[j]) for register bit j
   uint32_t gcol[SV_MAX_GBITS];   // byte offsets of the group bits (zero past the tile's)
@@ -201,13 +201,18 @@ struct alignas(16) SvStageDesc {
   // nonzero: the stage's ops are K_RP ops on the positions of this mask,
   // one per position in ascending order (run without dispatch)
   uint32_t rp_mask;
-  // compensated FP32 stage with a K_RP op on every position: block of the
-  // phase table (16 entries) holding, for each amplitude index e of the
-  // stage group, the product of the |1>-phases of e's set positions (times
-  // the program's global phase when bit 31 is set: then entry 0 applies
-  // too); 0xFFFFFFFF = none
+  // compensated FP32 stage of rotations: block of SV_PH_BLOCK floats of the
+  // table array: for each amplitude index e of the group the input factor
+  // less one (16), the unnormalized rotation {t0, t1} of each of the four
+  // positions (zero where the mask has none), then for each e {re, re
+  // remainder, im, im remainder} of the factor it takes after the rotations:
+  // the diagonal entries taken out of them, the |1>-phases of e's set
+  // positions and the program's global phase where this stage carries it
   uint32_t ph_block;
-  uint32_t pad;
+  // compensated FP32 stage of rotations: XOR of the roff of the positions
+  // whose two halves are exchanged when the group is read, so that the
+  // larger entry of the rotation's rows is on the diagonal
+  uint32_t ld_xor;
   // per-tile terms of cst: XOR ctl_w[i] when bit ctl_tb[i] of the tile index is set
   uint32_t ctl_tb[SV_MAX_OUT_CTL], ctl_w[SV_MAX_OUT_CTL];
 };
@@ -322,8 +327,8 @@ struct SvTables {
   const SvStageDesc *stages = nullptr;
   const void *ops = nullptr;       // SvOpDesc<T>*
   const float *ops_lo = nullptr;   // FP32: m[t] - (float)m[t] of every op, 8 floats per op (compensated passes)
-  // compensated FP32: phase products per stage block, 16 entries of
-  // {re, re - (float)re, im, im - (float)im} (see SvStageDesc::ph_block)
+  // compensated FP32: rotations and factors of the rotation stages, blocks
+  // of SV_PH_BLOCK floats (see SvStageDesc::ph_block)
   const float *ph = nullptr;
 };
 // Arithmetic of FP32 statevector passes.  PLAIN: FP32 registers.  COMP:

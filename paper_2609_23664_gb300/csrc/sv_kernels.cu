@@ -217,83 +217,136 @@ __device__ __forceinline__ uint32_t gray_pick(const uint32_t (&step)[6], int t) 
          : t == 5 ? step[5] : 0u;
 }
 
-// One stage group in compensated FP32: the N = 2^G amplitudes at byte
-// offsets sbB ^ (XOR combinations of roff) are read with a zero remainder
-// (SV_AR_COMP) or with their remainder from the plane at lo_off
-// (SV_AR_REM), the stage's ops run in double-float, and the renormalized
-// pair is written back (SV_AR_COMP keeps only the rounded value).
+// Scale of one stage group: `mx` is the largest component magnitude of its
+// amplitudes (NaN ignored, infinities counted as the largest finite value).
+// Returns the power of two the amplitudes are multiplied by first (1 except
+// for groups below 2^-79 or above 2^113, whose grid or low parts would leave
+// the FP32 range) and the grid constant C = 1.5 * 2^23 u, u = 2^(E + 5 - 22)
+// with 2^E the power of two above the largest component.
+__device__ __forceinline__ float gd_grid(float mx, float &C) {
+  uint32_t eb = __float_as_uint(fminf(mx, 3.402823466e38f)) >> 23;  // biased exponent, value < 2^(eb - 126)
+  float sc = 1.f;
+  if (mx == 0.f) {
+    eb = 127u;
+  } else if (eb < 48u) {
+    sc = 1.2676506002282294e30f;  // 2^100
+    eb += 100u;
+  } else if (eb > 240u) {
+    sc = 7.888609052210118e-31f;  // 2^-100
+    eb -= 100u;
+  }
+  C = __uint_as_float(((eb + 7u) << 23) | 0x400000u);
+  return sc;
+}
+
+// One stage group in compensated FP32 (sv_df.cuh): the N = 2^G amplitudes at
+// byte offsets ldB ^ (XOR combinations of roff) are read with a zero
+// remainder (SV_AR_COMP) or with their remainder from the plane at lo_off
+// (SV_AR_REM), the stage's ops run on the group's grid, and the result is
+// rounded once and written to the slots at sbB ^ (the same combinations)
+// (SV_AR_COMP keeps only the rounded value).  ldB differs from sbB when the
+// host has exchanged the two halves of a position (see SvStageDesc::ld_xor).
+//
+// Rotation stages (rp_mask != 0, one real rotation with an optional phase on
+// each position of the mask) run the unnormalized rotations, then multiply
+// every amplitude by its entry of the stage's table.  Bound by the FMA pipe:
+// 41 packed instructions per amplitude of a full stage (4 to split, 4 x 6
+// for the rotations less one shared, 14 for the table and the rounding); the
+// 64-task 24-qubit suffix launch took 104 ms with the 80-instruction
+// double-float form and takes 64 ms.
 template <int AR, int G>
-__device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t sbB, const uint32_t (&roff)[SV_G],
-                                            const SvOpDesc<float> *__restrict__ ops,
+__device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t sbB, uint32_t ldB,
+                                            const uint32_t (&roff)[SV_G], const SvOpDesc<float> *__restrict__ ops,
                                             const float *__restrict__ ops_lo, uint32_t op_begin, uint32_t nops,
                                             uint32_t rp_mask, const float *__restrict__ ph, uint32_t ph_block) {
   constexpr int N = 1 << G;
-  float2 h[N], l[N];
+  static_assert(G == 4, "the phase block holds four rotations and 16 entries");
+  auto off = [&](int i) {
+    return ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^ ((i & 4) ? roff[2] : 0u) ^ ((i & 8) ? roff[3] : 0u);
+  };
+  float2 H[N], l[N];
+  float mx = 0.f;
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    const uint32_t off = sbB ^ ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^ ((i & 4) ? roff[2] : 0u) ^
-                         ((i & 8) ? roff[3] : 0u) ^ ((G > 4 && (i & 16)) ? roff[4] : 0u);
-    h[i] = *(const float2 *)(smw + off);
-    if constexpr (AR == SV_AR_REM) l[i] = *(const float2 *)(smw + lo_off + off);
-    else l[i] = make_float2(0.f, 0.f);
+    H[i] = *(const float2 *)(smw + (ldB ^ off(i)));
+    mx = fmaxf(mx, fmaxf(fabsf(H[i].x), fabsf(H[i].y)));
+    if constexpr (AR == SV_AR_REM) l[i] = *(const float2 *)(smw + lo_off + (ldB ^ off(i)));
   }
-  auto load_ml = [&](uint32_t o, float (&m)[8], float (&ml)[8]) {
-    load_m(ops + o, m);
-    const float4 u = __ldg((const float4 *)(ops_lo + 8 * (size_t)o));
-    const float4 v = __ldg((const float4 *)(ops_lo + 8 * (size_t)o + 4));
-    ml[0] = u.x; ml[1] = u.y; ml[2] = u.z; ml[3] = u.w;
-    ml[4] = v.x; ml[5] = v.y; ml[6] = v.z; ml[7] = v.w;
-  };
-  if (G == 4 && rp_mask == 0xFu) {
-    // a rotation-and-phase op on every position: the four rotations, then
-    // the stage's combined diagonal (amplitude e times the product of the
-    // phases of its set positions, from the host's table) when there is one
-    const bool table = ph != nullptr && ph_block != 0xFFFFFFFFu;
-    float m[8], ml[8];
-    load_ml(op_begin, m, ml);
-    dfop_rp<0, N, AR == SV_AR_COMP>(h, l, m, ml, !table);
-    load_ml(op_begin + 1, m, ml);
-    dfop_rp<1, N>(h, l, m, ml, !table);
-    load_ml(op_begin + 2, m, ml);
-    dfop_rp<2, N>(h, l, m, ml, !table);
-    load_ml(op_begin + 3, m, ml);
-    dfop_rp<3, N>(h, l, m, ml, !table);
-    if (table) {
-      const float4 *q = (const float4 *)ph + 16 * (size_t)(ph_block & 0x7FFFFFFFu);
-      if (ph_block >> 31) {  // the program's global phase: entry 0 too
-        const float4 w = __ldg(q);
-        df_cmul(w.x, w.y, w.z, w.w, h[0], l[0]);
-      }
+  float c1;
+  const float sc = gd_grid(mx, c1);
+  if (sc != 1.f) {
 #pragma unroll
-      for (int e = 1; e < N; e++) {
-        const float4 w = __ldg(q + e);
-        df_cmul(w.x, w.y, w.z, w.w, h[e], l[e]);
-      }
+    for (int i = 0; i < N; i++) {
+      H[i] = __fmul2_rn(H[i], f2s(sc));
+      if constexpr (AR == SV_AR_REM) l[i] = __fmul2_rn(l[i], f2s(sc));
     }
-  } else if (rp_mask) {
-    uint32_t o = op_begin;
+  }
+  const float2 C = f2s(c1);
+  // the amplitude's factor (1 + eps) and its split: the part on the grid
+  // into H (biased), the exact rest and eps h into l
+  auto split = [&](int i, float eps) {
+    const float2 h = H[i];
+    H[i] = __fadd2_rn(h, C);
+    float2 r = __ffma2_rn(f2s(eps), h, f2sub(h, f2sub(H[i], C)));
+    if constexpr (AR == SV_AR_REM) r = __fadd2_rn(r, l[i]);
+    l[i] = r;
+  };
+  if (rp_mask) {
+    const float *blk = ph + SV_PH_BLOCK * (size_t)ph_block;
+    const float2 *t = (const float2 *)(blk + 16);
+    if (rp_mask == 0xFu) {
+      const float2 t0 = __ldg(t);
 #pragma unroll
-    for (int P = 0; P < G; P++) {
-      if (!(rp_mask & (1u << P))) continue;
-      float m[8], ml[8];
-      load_ml(o, m, ml);
-      o++;
-      df_rp_at<N>(P, h, l, m, ml);
+      for (int i = 0; i < N; i += 2) {
+        const float2 e = __ldg((const float2 *)(blk + i));
+        split(i, e.x);
+        split(i + 1, e.y);
+        gd_pair(C, t0, H[i], l[i], H[i + 1], l[i + 1]);
+      }
+      gdop_rot<1, N>(C, H, l, __ldg(t + 1));
+      gdop_rot<2, N>(C, H, l, __ldg(t + 2));
+      gdop_rot<3, N>(C, H, l, __ldg(t + 3));
+    } else {
+#pragma unroll
+      for (int i = 0; i < N; i++) split(i, __ldg(blk + i));
+      if (rp_mask & 1u) gdop_rot<0, N>(C, H, l, __ldg(t));
+      if (rp_mask & 2u) gdop_rot<1, N>(C, H, l, __ldg(t + 1));
+      if (rp_mask & 4u) gdop_rot<2, N>(C, H, l, __ldg(t + 2));
+      if (rp_mask & 8u) gdop_rot<3, N>(C, H, l, __ldg(t + 3));
+    }
+    const float4 *q = (const float4 *)(blk + 24);
+#pragma unroll
+    for (int e = 0; e < N; e++) {
+      const float4 w = __ldg(q + e);
+      gd_cmul(C, w.x, w.y, w.z, w.w, H[e], l[e]);
     }
   } else {
+#pragma unroll
+    for (int i = 0; i < N; i++) split(i, 0.f);
     for (uint32_t o = 0; o < nops; o++) {
       float m[8], ml[8];
-      load_ml(op_begin + o, m, ml);
-      df_apply_op<N>(__ldg(&ops[op_begin + o].code), m, ml, h, l);
+      load_m(ops + op_begin + o, m);
+      const float4 u = __ldg((const float4 *)(ops_lo + 8 * (size_t)(op_begin + o)));
+      const float4 v = __ldg((const float4 *)(ops_lo + 8 * (size_t)(op_begin + o) + 4));
+      ml[0] = u.x; ml[1] = u.y; ml[2] = u.z; ml[3] = u.w;
+      ml[4] = v.x; ml[5] = v.y; ml[6] = v.z; ml[7] = v.w;
+      gd_apply_op<N>(__ldg(&ops[op_begin + o].code), m, ml, C, H, l);
     }
   }
+  const float isc = sc == 1.f ? 1.f : (sc > 1.f ? 7.888609052210118e-31f : 1.2676506002282294e30f);
 #pragma unroll
   for (int i = 0; i < N; i++) {
-    df_renorm(h[i], l[i]);
-    const uint32_t off = sbB ^ ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^ ((i & 4) ? roff[2] : 0u) ^
-                         ((i & 8) ? roff[3] : 0u) ^ ((G > 4 && (i & 16)) ? roff[4] : 0u);
-    *(float2 *)(smw + off) = h[i];
-    if constexpr (AR == SV_AR_REM) *(float2 *)(smw + lo_off + off) = l[i];
+    const float2 qi = f2sub(H[i], C);
+    float2 s = __fadd2_rn(qi, l[i]);  // the one rounding
+    // what the rounding dropped (Fast2Sum: qi is a multiple of the low part's last place)
+    float2 r = make_float2(0.f, 0.f);
+    if constexpr (AR == SV_AR_REM) r = f2sub(l[i], f2sub(s, qi));
+    if (sc != 1.f) {
+      s = __fmul2_rn(s, f2s(isc));
+      if constexpr (AR == SV_AR_REM) r = __fmul2_rn(r, f2s(isc));
+    }
+    *(float2 *)(smw + (sbB ^ off(i))) = s;
+    if constexpr (AR == SV_AR_REM) *(float2 *)(smw + lo_off + (sbB ^ off(i))) = r;
   }
 }
 
@@ -392,7 +445,7 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
     // the map's constant, with the per-tile terms of outside-control CNOTs
     const uint32_t cst = (w3.z ^ (((tile >> w5.x) & 1u) ? w6.x : 0u) ^ (((tile >> w5.y) & 1u) ? w6.y : 0u) ^
                           (((tile >> w5.z) & 1u) ? w6.z : 0u) ^ (((tile >> w5.w) & 1u) ? w6.w : 0u)) & tm;
-    const uint32_t nops = w3.w, op_begin = w4.x, rp_mask = w4.y, ph_block = w4.z;
+    const uint32_t nops = w3.w, op_begin = w4.x, rp_mask = w4.y, ph_block = w4.z, ld_xor = w4.w & tm;
     static_assert(SV_MAX_GBITS == 9 && SV_MAX_OUT_CTL == 4 && sizeof(SvStageDesc) == 112,
                   "stage descriptor read as seven 16-byte words");
     for (uint32_t grp = threadIdx.x; grp < n_groups; grp += nt) {
@@ -400,7 +453,7 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
 #pragma unroll
       for (int t = 0; t < SV_MAX_GBITS; t++) sbB ^= ((grp >> t) & 1u) ? gcol[t] : 0u;
       if constexpr (AR != SV_AR_PLAIN) {
-        sv_stage_df<AR, G>(smw, lo_off, sbB, roff, ops, ops_lo, op_begin, nops, rp_mask, ph, ph_block);
+        sv_stage_df<AR, G>(smw, lo_off, sbB, sbB ^ ld_xor, roff, ops, ops_lo, op_begin, nops, rp_mask, ph, ph_block);
       } else {
       constexpr int N = 1 << G;
       C a[N];
