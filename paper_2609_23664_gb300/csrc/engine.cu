@@ -396,7 +396,6 @@ struct DeviceState {
   std::vector<void *> mat_buf;
   std::vector<void *> mat_export[2];   // per mode (FP64, FP32): statevector exported from a tableau node
   std::vector<StabBasis *> mat_basis;  // scratch of each exporting tableau node
-  std::vector<int> tab_launch_of_mat;  // index into tab_mat_launches, -1 none
   std::vector<qw_dense_prog *> mat_dense;  // boundary evolved by a dense-block program, else NULL
   // statevector boundaries of one precision in one persistent launch (a
   // boundary's first pass waits for its parent's last); empty = per-pass launches
@@ -1126,19 +1125,15 @@ static void prepare(qw_plan *P) {
     for (size_t m = 0; m < P->mats.size(); m++) P->outs_mat_off[m + 1] = P->outs_mat_off[m] + P->mats[m].tab_outs;
     D->d_outs = (uint8_t *)D->arena.alloc(std::max<uint32_t>(1, P->outs_off[nt]));
     D->d_mat_outs = (uint8_t *)D->arena.alloc(std::max<uint32_t>(1, P->outs_mat_off[P->mats.size()]));
-    auto add_launch = [&](std::vector<DeviceState::TabLaunch> &dst, uint32_t n, const void *init,
-                          void *out_buf, const std::vector<TabTaskDesc> &descs,
+    auto sign_of = [](uint64_t *rows, uint32_t n) {
+      return rows ? (uint8_t *)(rows + (size_t)2 * n * 2 * ((n + 63) / 64)) : nullptr;
+    };
+    auto add_launch = [&](std::vector<DeviceState::TabLaunch> &dst, uint32_t n, const std::vector<TabTaskDesc> &descs,
                           const std::vector<TabSegment> &segs, uint8_t *outs) {
       TabArgs a{};
       a.n = n;
       a.W = (n + 63) / 64;
-      a.lpp = a.W <= 8 ? 8 : (a.W <= 16 ? 16 : 32);
       a.rows = 2 * n;
-      const size_t words = (size_t)a.rows * 2 * a.W;
-      a.init_rows = (const uint64_t *)init;
-      a.init_sign = init ? (const uint8_t *)((const uint64_t *)init + words) : nullptr;
-      a.out_rows = (uint64_t *)out_buf;
-      a.out_sign = out_buf ? (uint8_t *)((uint64_t *)out_buf + words) : nullptr;
       a.tasks = D->arena.upload(descs, s);
       a.segs = D->arena.upload(segs, s);
       a.progs = D->d_progs;
@@ -1148,58 +1143,74 @@ static void prepare(qw_plan *P) {
       a.outs = outs;
       dst.push_back({a, (uint32_t)descs.size(), -1});
     };
-    D->tab_launch_of_mat.assign(P->mats.size(), -1);
-    for (size_t m = 0; m < P->mats.size(); m++) {
-      const MatNode &M = P->mats[m];
-      if (M.mode != QW_MODE_TABLEAU) continue;
-      D->tab_launch_of_mat[m] = (int)D->tab_mat_launches.size();
-      std::vector<TabSegment> segs;
+    // appends one CTA: its segments (outcomes relative to out_base) and descriptor
+    auto add_desc = [&](std::vector<TabTaskDesc> &descs, std::vector<TabSegment> &segs,
+                        const std::vector<std::pair<uint32_t, uint32_t>> &tab_segs, uint32_t out_base,
+                        const void *init, uint64_t *out_rows, uint8_t *out_sign) {
+      TabTaskDesc d{};
+      d.seg_begin = (uint32_t)segs.size();
+      d.n_segs = (uint32_t)tab_segs.size();
+      d.out_base = out_base;
+      d.init_rows = (const uint64_t *)init;
+      d.out_rows = out_rows;
+      d.out_sign = out_sign;
       uint32_t oo = 0;
-      for (auto &sg : M.tab_segs) {
+      for (auto &sg : tab_segs) {
         segs.push_back({sg.first, sg.second, oo, 0});
         oo += P->tab_progs[sg.first].n_outs;
       }
-      std::vector<TabTaskDesc> d{{0, (uint32_t)segs.size(), 0, P->outs_mat_off[m]}};
-      add_launch(D->tab_mat_launches, M.n, M.parent >= 0 ? D->mat_buf[M.parent] : nullptr,
-                 D->mat_buf[m], d, segs, D->d_mat_outs);
+      descs.push_back(d);
+    };
+    // Boundaries: every boundary of one register size whose parent is ready
+    // runs in one launch, a CTA each (level by level; parents precede their
+    // children in the list).  A launch per boundary left one SM busy at a
+    // time: 129 boundaries of a random-outcome workload took 129 launches.
+    {
+      std::vector<uint32_t> level(P->mats.size(), 0);
+      std::map<std::pair<uint32_t, uint32_t>, std::vector<size_t>> by_level;  // (level, n) -> boundaries
+      for (size_t m = 0; m < P->mats.size(); m++) {
+        const MatNode &M = P->mats[m];
+        if (M.mode != QW_MODE_TABLEAU) continue;
+        if (M.parent >= 0) level[m] = level[M.parent] + 1;
+        by_level[{level[m], M.n}].push_back(m);
+      }
+      for (auto &lv : by_level) {
+        std::vector<TabTaskDesc> descs;
+        std::vector<TabSegment> segs;
+        const uint32_t n = lv.first.second;
+        for (size_t m : lv.second) {
+          const MatNode &M = P->mats[m];
+          uint64_t *out = (uint64_t *)D->mat_buf[m];
+          add_desc(descs, segs, M.tab_segs, P->outs_mat_off[m], M.parent >= 0 ? D->mat_buf[M.parent] : nullptr, out,
+                   sign_of(out, n));
+        }
+        add_launch(D->tab_mat_launches, n, descs, segs, D->d_mat_outs);
+      }
     }
+    // Tasks: those of one register size run in one launch, each from its own
+    // boundary, except Pauli-frame groups, whose launch is gated by their
+    // own reference run
     std::map<std::pair<int, uint32_t>, std::vector<uint32_t>> by_src;
     for (uint32_t t = 0; t < nt; t++)
-      if (P->tasks[t].mode == QW_MODE_TABLEAU) by_src[{P->tasks[t].src, P->tasks[t].n}].push_back(t);
+      if (P->tasks[t].mode == QW_MODE_TABLEAU)
+        by_src[{P->task_frame_group[t] >= 0 ? P->tasks[t].src : -1, P->tasks[t].n}].push_back(t);
     D->tab_keep.assign(nt, {nullptr, nullptr});
     for (auto &g : by_src) {
       std::vector<TabTaskDesc> descs;
       std::vector<TabSegment> segs;
+      const uint32_t kn = g.first.second;
+      const size_t kwords = (size_t)2 * kn * 2 * ((kn + 63) / 64);
       for (uint32_t t : g.second) {
         const TaskPlan &tp = P->tasks[t];
-        TabTaskDesc d{};
-        d.seg_begin = (uint32_t)segs.size();
-        d.out_base = P->outs_off[t];
-        uint32_t oo = 0;
-        for (auto &sg : tp.tab_segs) {
-          segs.push_back({sg.first, sg.second, oo, 0});
-          oo += P->tab_progs[sg.first].n_outs;
+        uint64_t *keep = nullptr;  // final tableau of a task that keeps its state
+        if (tp.flags & QW_TASK_KEEP_STATE) {
+          keep = (uint64_t *)D->arena.alloc(kwords * 8 + 2 * kn);
+          D->tab_keep[t] = {keep, sign_of(keep, kn)};
         }
-        d.n_segs = (uint32_t)segs.size() - d.seg_begin;
-        descs.push_back(d);
+        add_desc(descs, segs, tp.tab_segs, P->outs_off[t], tp.src >= 0 ? D->mat_buf[tp.src] : nullptr, keep,
+                 sign_of(keep, kn));
       }
-      // tasks that keep their final tableau: the whole launch writes its
-      // tableaus back (rows of every task, then the signs of every task)
-      bool keep = false;
-      for (uint32_t t : g.second) keep = keep || (P->tasks[t].flags & QW_TASK_KEEP_STATE);
-      void *keep_buf = nullptr;
-      const uint32_t kn = g.first.second, kW = (kn + 63) / 64;
-      const size_t kwords = (size_t)2 * kn * 2 * kW, nk = g.second.size();
-      if (keep) keep_buf = D->arena.alloc(nk * (kwords * 8 + 2 * kn));
-      add_launch(D->tab_task_launches, g.first.second,
-                 g.first.first >= 0 ? D->mat_buf[g.first.first] : nullptr, keep_buf, descs, segs,
-                 D->d_outs);
-      if (keep) {
-        uint8_t *signs = (uint8_t *)((uint64_t *)keep_buf + nk * kwords);
-        D->tab_task_launches.back().a.out_sign = signs;
-        for (size_t k = 0; k < nk; k++)
-          D->tab_keep[g.second[k]] = {(const uint64_t *)keep_buf + k * kwords, signs + k * 2 * kn};
-      }
+      add_launch(D->tab_task_launches, kn, descs, segs, D->d_outs);
       const int fg = P->task_frame_group[g.second[0]];
       if (fg >= 0) {
         // Pauli frames: the reference suffix once on the tableau, then the
@@ -1210,14 +1221,10 @@ static void prepare(qw_plan *P) {
         uint8_t *ref_out = (uint8_t *)D->arena.alloc(std::max<uint32_t>(1, G.n_outs));
         uint32_t *rand = (uint32_t *)D->arena.alloc(sizeof(uint32_t));
         std::vector<TabSegment> rsegs;
-        uint32_t oo = 0;
-        for (auto &sg : G.ref_segs) {
-          rsegs.push_back({sg.first, sg.second, oo, 0});
-          oo += P->tab_progs[sg.first].n_outs;
-        }
-        std::vector<TabTaskDesc> rd{{0, (uint32_t)rsegs.size(), 0, 0}};
+        std::vector<TabTaskDesc> rd;
+        add_desc(rd, rsegs, G.ref_segs, 0, D->mat_buf[G.src], nullptr, nullptr);
         std::vector<DeviceState::TabLaunch> tmp;
-        add_launch(tmp, G.n, D->mat_buf[G.src], nullptr, rd, rsegs, ref_out);
+        add_launch(tmp, G.n, rd, rsegs, ref_out);
         DeviceState::FrameLaunch fl{};
         fl.ref = tmp[0].a;
         fl.ref.rand_any = rand;
@@ -1260,13 +1267,15 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
     return capturing ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal) : cudaEventRecord(e, s);
   };
   CK(rec(D->ev[0]));
-  // 1) shared prefixes (boundary states), in creation order (parents first)
+  // 1) shared prefixes (boundary states): the tableaus level by level, then
+  // the statevectors in creation order (parents first)
+  for (const DeviceState::TabLaunch &L : D->tab_mat_launches) {
+    launch_tab(L.a, L.n_tasks, s);
+    nl += 1;
+  }
   for (size_t m = 0; m < P->mats.size(); m++) {
     const MatNode &M = P->mats[m];
     if (M.mode == QW_MODE_TABLEAU) {
-      const DeviceState::TabLaunch &L = D->tab_mat_launches[D->tab_launch_of_mat[m]];
-      launch_tab(L.a, L.n_tasks, s);
-      nl += 1;
       // Table II STAB -> SV: the statevectors its consumers continue from
       for (uint32_t md = 0; md < 2; md++)
         if (D->mat_export[md][m]) {

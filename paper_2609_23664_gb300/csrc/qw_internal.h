@@ -301,10 +301,14 @@ struct TabProgram {
 struct TabSegment {
   uint32_t prog, bit_base, out_base, pad;
 };
+// one CTA of a tableau launch
 struct TabTaskDesc {
   uint32_t seg_begin, n_segs;
-  uint32_t bits_base;   // into the byte array of random bits
-  uint32_t out_base;    // into the outcome byte array
+  uint32_t bits_base;         // into the byte array of random bits
+  uint32_t out_base;          // into the outcome byte array
+  const uint64_t *init_rows;  // boundary tableau, its rows followed by its signs (NULL = identity)
+  uint64_t *out_rows;         // final tableau written back when non-NULL
+  uint8_t *out_sign;
 };
 struct TabHostProgram {
   std::vector<TabLayer> layers;
@@ -405,11 +409,7 @@ void launch_sampling(bool fp64, const SmpSource *srcs, uint32_t n_src, uint32_t 
 
 // tableau
 struct TabArgs {
-  uint32_t n, W, lpp, rows;
-  const uint64_t *init_rows;   // boundary tableau (NULL = identity)
-  const uint8_t *init_sign;
-  uint64_t *out_rows;          // written back when non-NULL (boundary producer)
-  uint8_t *out_sign;
+  uint32_t n, W, rows;
   const TabTaskDesc *tasks;
   const TabSegment *segs;
   const TabProgram *progs;
