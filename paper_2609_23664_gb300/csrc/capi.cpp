@@ -365,7 +365,10 @@ qw_status qw_get_samples(const qw_plan *p, uint64_t task, uint64_t *out, size_t 
   QW_GUARD({
     const TaskPlan &tp = task_of(p, task);
     if (n) *n = tp.shots;
-    if (cap < tp.shots) fail(QW_ERR_BUFFER_TOO_SMALL, "need %u entries", tp.shots);
+    if (cap < tp.shots) {  // the sizing call: answered without an exception
+      set_last_error(strf("need %u entries", tp.shots));
+      return QW_ERR_BUFFER_TOO_SMALL;
+    }
     if (tp.shots && !out) fail(QW_ERR_INVALID_ARG, "out is NULL");
     std::copy(p->samples.begin() + p->sample_off[task], p->samples.begin() + p->sample_off[task + 1], out);
   })
@@ -376,17 +379,23 @@ qw_status qw_get_syndrome(const qw_plan *p, uint64_t task, uint8_t *bits, size_t
     const TaskPlan &tp = task_of(p, task);
     if (tp.mode != QW_MODE_TABLEAU) fail(QW_ERR_NOT_FOUND, "task %llu is not a tableau task", (unsigned long long)task);
     if (n_bits) *n_bits = tp.total_outs;
-    if (cap < tp.total_outs) fail(QW_ERR_BUFFER_TOO_SMALL, "need %u bytes", tp.total_outs);
-    if (tp.total_outs && !bits) fail(QW_ERR_INVALID_ARG, "bits is NULL");
-    // outcomes of the materialized chain from the root, then the task's own
-    std::vector<int> chain;
-    for (int m = tp.src; m >= 0; m = p->mats[m].parent) chain.push_back(m);
-    size_t o = 0;
-    for (auto it = chain.rbegin(); it != chain.rend(); ++it) {
-      const int m = *it;
-      for (uint32_t i = p->outs_mat_off[m]; i < p->outs_mat_off[m + 1]; i++) bits[o++] = p->outs_mat[i];
+    if (cap < tp.total_outs) {  // the sizing call of every reader: answered without an exception
+      set_last_error(strf("need %u bytes", tp.total_outs));
+      return QW_ERR_BUFFER_TOO_SMALL;
     }
-    for (uint32_t i = p->outs_off[task]; i < p->outs_off[task + 1]; i++) bits[o++] = p->outs_suffix[i];
+    if (tp.total_outs && !bits) fail(QW_ERR_INVALID_ARG, "bits is NULL");
+    if (tp.total_outs == 0) return QW_OK;
+    // outcomes of the materialized chain from the root, then the task's own
+    // (block copies, from the end backwards: a task of 105 surface-code
+    // rounds returns 23 KB)
+    const size_t own = p->outs_off[task + 1] - p->outs_off[task];
+    size_t o = tp.total_outs - own;
+    if (own) memcpy(bits + o, p->outs_suffix.data() + p->outs_off[task], own);
+    for (int m = tp.src; m >= 0; m = p->mats[m].parent) {
+      const size_t k = p->outs_mat_off[m + 1] - p->outs_mat_off[m];
+      o -= k;
+      if (k) memcpy(bits + o, p->outs_mat.data() + p->outs_mat_off[m], k);
+    }
   })
 }
 

@@ -329,20 +329,23 @@ class Plan:
         _check(lib().qw_get_energy(self.h, t, C.byref(e), C.byref(n)))
         return e.value, n.value
 
+    # result arrays: the size from a call without a buffer, then the values
+    # (the second call writes every element)
     def samples(self, t: int) -> np.ndarray:
+        fn = lib().qw_get_samples
         n = C.c_size_t()
-        st = lib().qw_get_samples(self.h, t, None, 0, C.byref(n))
-        out = np.zeros(n.value, dtype=np.uint64)
-        if n.value == 0:
-            return out
-        _check(lib().qw_get_samples(self.h, t, _p(out), len(out), C.byref(n)))
+        fn(self.h, t, None, 0, C.byref(n))
+        out = np.empty(n.value, dtype=np.uint64)
+        if n.value:
+            _check(fn(self.h, t, out.ctypes.data, n.value, None))
         return out
 
     def syndrome(self, t: int) -> np.ndarray:
+        fn = lib().qw_get_syndrome
         n = C.c_size_t()
-        lib().qw_get_syndrome(self.h, t, None, 0, C.byref(n))
-        out = np.zeros(n.value, dtype=np.uint8)
-        _check(lib().qw_get_syndrome(self.h, t, _p(out) if n.value else None, len(out), C.byref(n)))
+        fn(self.h, t, None, 0, C.byref(n))
+        out = np.empty(n.value, dtype=np.uint8)
+        _check(fn(self.h, t, out.ctypes.data if n.value else None, n.value, None))
         return out
 
     def state(self, t: int, n: int, fp64: bool) -> np.ndarray:
