@@ -472,9 +472,9 @@ qw_status qw_sv_sample_dev(qw_engine *e, uint32_t mode, uint32_t n, const void *
  * computes what qw_sv_energy_dev computes, with the same kernels, but needs
  * no engine and allocates nothing: the term layout, the job record and the
  * per-block partial sums live in one fixed device array of the library
- * (about 1.2 MB, held by every GPU that loads the library until the process
- * exits).  Its term classes are fixed (chunks of an eighth of the state from
- * 15 qubits on), so its sums run in another order than qw_sv_energy_dev's.
+ * (about 1.1 MB, held by every GPU that loads the library until the process
+ * exits).  Its term layout is bounded (at most 8 classes of terms), so above
+ * 25 FP32 qubits its sums run in another order than qw_sv_energy_dev's.
  *   state : device, 2^n amplitudes (double2 for QW_MODE_SV_FP64, float2 for
  *           QW_MODE_SV_FP32), n in [5, QW_NOALLOC_MAX_QUBITS].
  *   terms : host, n_terms <= QW_NOALLOC_MAX_TERMS; masks within n bits.

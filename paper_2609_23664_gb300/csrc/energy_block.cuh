@@ -1,23 +1,27 @@
 // Pauli-sum energy over one block of amplitudes, shared by the stand-alone
-// energy kernel (256 threads) and by the persistent suffix kernel, which
-// runs energy blocks as a second kind of work item (128 threads, two
-// sub-blocks per 4096-amplitude block).
+// energy kernel and by the persistent suffix kernel, which runs energy
+// blocks as a second kind of work item.
 //
 // E = sum_k c_k <psi|P_k|psi> / <psi|psi>, P|x> = i^{#Y} (-1)^{popc(x&z)}|x^m>.
-// For m != 0 the pair (x, x^m) is visited once from the side whose highest
-// flipped bit is 0 and contributes 2 Re(i^{#Y} (-1)^{popc(x&z)}
-// conj(psi[x^m]) psi[x]); the host folds 2, the sign of i^{#Y} and the
-// coefficient into EnTerm::coef and the choice of real or imaginary part into
-// EnTerm::flags.  Terms are grouped into classes by the flipped bits above an
-// L2-sized chunk, so the blocks of one class read one pair of chunks.
+// For m != 0 the pair (x, x^m) is visited once and contributes
+// 2 Re(i^{#Y} (-1)^{popc(x&z)} conj(psi[x^m]) psi[x]); the host folds 2, the
+// sign of i^{#Y} and the coefficient into EnTerm::coef and the choice of real
+// or imaginary part into EnTerm::code.
 //
-// A sub-block holds 16 << TB amplitudes; element j of thread t has index
-// x = base | j << TB | t.  The three fields are disjoint bit ranges, so for
-// a term (m, z) the partner of element j is pb | (j ^ mj) << TB with pb the
-// partner of element 0, and its sign is (-1)^{popc((base|t) & z)} times
-// (-1)^{popc(j & zj)}.  The partner offsets are resolved at compile time by
-// a switch over (mj, flags), so a partner load is one load with an immediate
-// offset; the signs are applied by a branch-free butterfly.
+// Terms are evaluated in groups of up to four independent flip masks.  With V
+// the span of a group's masks, a thread loads the 16 amplitudes of one coset
+// x0 ^ V into registers, where every pair of every term whose mask lies in V
+// is at hand: the state is read once per four terms instead of half of it
+// once per term, which halves the L2 -> SM traffic that bounds the kernel
+// (200 random terms at 24 qubits: 52 sweeps of the state, 6.7 GB, instead of
+// 14 GB; the SMs take at most 64 bytes per clock each from L2).
+//
+// A coset is represented by its element with zeros at the pivot bits of V
+// (its leading bits), so consecutive representatives are consecutive
+// addresses except at the pivots and a warp's loads stay coalesced.  Groups
+// are formed within a class of terms that flip the same bits above an
+// L2-sized chunk: the blocks of one class then sweep one pair of chunks at a
+// time, which stays in L2 while all groups of the class visit it.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -50,6 +54,27 @@ template <typename T> struct AccOf;
 template <> struct AccOf<float> { typedef DFAcc t; };
 template <> struct AccOf<double> { typedef DAcc t; };
 
+// Warp sums of the lanes' accumulators and of their norms.  FP32 blocks add
+// in double-float: FP64 adds run at 1/64 of the FP32 rate, and a block is
+// short enough (13 groups per class) that 12 of them per thread showed.
+__device__ __forceinline__ double en_warp_total(DFAcc a) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
+    a.add(h);
+    a.lo += l;
+  }
+  return a.value();
+}
+__device__ __forceinline__ double en_warp_sum(double v);
+__device__ __forceinline__ double en_warp_total(DAcc a) { return en_warp_sum(a.v); }
+__device__ __forceinline__ double en_warp_total_norm(float v) {
+  DFAcc a;
+  a.hi = v;
+  return en_warp_total(a);
+}
+__device__ __forceinline__ double en_warp_total_norm(double v) { return en_warp_sum(v); }
+
 __device__ __forceinline__ double en_warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -65,141 +90,246 @@ __device__ __forceinline__ C en_ld(const C *p) {
   return __ldcg(p);
 }
 
-// sum_j (-1)^{popc(j & z)} v[j] as a butterfly over the four bits of j with
-// runtime signs: 15 fused multiply-adds by +-1 (exact products), no branch
-template <typename T>
-__device__ __forceinline__ T en_signed16_bf(const T (&v)[16], uint32_t z) {
-  const T s0 = (z & 1u) ? T(-1) : T(1), s1 = (z & 2u) ? T(-1) : T(1);
-  const T s2 = (z & 4u) ? T(-1) : T(1), s3 = (z & 8u) ? T(-1) : T(1);
-  T u[8], w[4];
-#pragma unroll
-  for (int k = 0; k < 8; k++) u[k] = fma(s0, v[2 * k + 1], v[2 * k]);
-#pragma unroll
-  for (int k = 0; k < 4; k++) w[k] = fma(s1, u[2 * k + 1], u[2 * k]);
-  const T x0 = fma(s2, w[1], w[0]), x1 = fma(s2, w[3], w[2]);
-  return fma(s3, x1, x0);
+// Amplitudes of a thread: index i = combination of the four basis masks, and
+// below it in FP32 blocks of aligned states (PAIR) the two neighbours 2x, 2x+1
+// that one 16-byte load brings: the span then has bit 0 as a fifth direction,
+// and everything that is per thread and term (addresses, signs, branches) is
+// paid once for 32 amplitudes.
+template <typename T, bool PAIR> struct EnAmp {
+  typedef typename EnC<T>::t C;
+  static constexpr int N = PAIR ? 32 : 16;
+};
+
+// k-th pair {x, x ^ m} for m = basis combination MC, and bit 0 when E (PAIR):
+// index of its first member, whose highest flipped direction is clear
+template <int MC, int E, bool PAIR>
+__device__ __forceinline__ constexpr int en_low(int k) {
+  constexpr int m = PAIR ? 2 * MC + E : MC;
+  constexpr int h = m >= 16 ? 4 : m >= 8 ? 3 : m >= 4 ? 2 : m >= 2 ? 1 : 0;
+  return m ? (((k >> h) << (h + 1)) | (k & ((1 << h) - 1))) : k;
 }
 
-// v[j] = Re or Im part of conj(partner_j) a[j], partner_j = q[(j ^ MJ) << TB]
-template <typename T, int TB, bool NC, int MJ, bool FL, typename C>
-__device__ __forceinline__ void en_prod(const C *__restrict__ q, const C (&a)[16], T (&v)[16]) {
-  C p[16];
+// Sum over those pairs of (-1)^{popc(x & z)} times the real (IM: imaginary)
+// part of conj(a[x ^ m]) a[x]; m = 0: over all amplitudes, with |a[x]|^2.
+// FP32 adds through a butterfly of +-1 multiply-adds (exact products, no
+// branch) with the signs s of the pair index's bits, the real part on both
+// components at once (packed instructions: the kernel is bound by
+// instruction issue); FP64, whose pipe runs at 1/64 of the FP32 rate, flips
+// signs on the integer pipe instead and accumulates straight into its
+// multiply-adds (16 FP64 operations per 8 pairs, not 23).
+template <int MC, int E, bool IM, bool PAIR>
+__device__ __forceinline__ float en_pairs(const float2 (&a)[EnAmp<float, PAIR>::N], const float (&s)[5]) {
+  constexpr int m = PAIR ? 2 * MC + E : MC, N = EnAmp<float, PAIR>::N, NP = m ? N / 2 : N;
+  if constexpr (IM) {
+    float v[NP];
 #pragma unroll
-  for (int j = 0; j < 16; j++) p[j] = en_ld<NC>(q + ((j ^ MJ) << TB));
+    for (int k = 0; k < NP; k++) {
+      const float2 x = a[en_low<MC, E, PAIR>(k)], p = a[en_low<MC, E, PAIR>(k) ^ m];
+      v[k] = p.x * x.y - p.y * x.x;
+    }
 #pragma unroll
-  for (int j = 0; j < 16; j++)
-    v[j] = FL ? (p[j].x * a[j].y - p[j].y * a[j].x) : (p[j].x * a[j].x + p[j].y * a[j].y);
+    for (int w = NP / 2, b = 0; w > 0; w /= 2, b++)
+#pragma unroll
+      for (int k = 0; k < w; k++) v[k] = fmaf(s[b], v[2 * k + 1], v[2 * k]);
+    return v[0];
+  } else {
+    float2 v[NP];
+#pragma unroll
+    for (int k = 0; k < NP; k++) v[k] = __fmul2_rn(a[en_low<MC, E, PAIR>(k) ^ m], a[en_low<MC, E, PAIR>(k)]);
+#pragma unroll
+    for (int w = NP / 2, b = 0; w > 0; w /= 2, b++) {
+      const float2 sb = make_float2(s[b], s[b]);
+#pragma unroll
+      for (int k = 0; k < w; k++) v[k] = __ffma2_rn(sb, v[2 * k + 1], v[2 * k]);
+    }
+    return v[0].x + v[0].y;
+  }
 }
-template <typename T, int TB, bool NC, typename C>
-__device__ __forceinline__ void en_prod_rt(const C *__restrict__ q, const C (&a)[16], T (&v)[16],
-                                           uint32_t sel) {
-  switch (sel & 31u) {
-#define QW_PR(S) case S: en_prod<T, TB, NC, (S & 15), (S >= 16)>(q, a, v); break;
+template <int MC, int E, bool IM, bool PAIR>
+__device__ __forceinline__ double en_pairs(const double2 (&a)[16], uint32_t zz) {
+  static_assert(!PAIR, "FP64 amplitudes are 16 bytes each");
+  double s0 = 0, s1 = 0;
+#pragma unroll
+  for (int k = 0; k < (MC ? 8 : 16); k++) {
+    const int i = en_low<MC, 0, false>(k);
+    const int sgn = (__popc((uint32_t)i & zz) & 1) << 31;
+    const double2 p = a[i ^ MC];
+    const double px = __hiloint2double(__double2hiint(p.x) ^ sgn, __double2loint(p.x));
+    const double py = __hiloint2double(__double2hiint(p.y) ^ sgn, __double2loint(p.y));
+    s0 = fma(px, IM ? a[i].y : a[i].x, s0);
+    s1 = fma(IM ? -py : py, IM ? a[i].x : a[i].y, s1);
+  }
+  return s0 + s1;
+}
+// the term's sign data in the form its precision takes
+template <typename T> struct EnSign;
+template <> struct EnSign<float> {
+  float s[5];
+  __device__ __forceinline__ EnSign(const EnTerm *t, uint32_t code) {
+    const float4 v = __ldg((const float4 *)t + 1);
+    s[0] = v.x; s[1] = v.y; s[2] = v.z; s[3] = v.w;
+    s[4] = (code & EN_LAST_SIGN) ? -1.f : 1.f;  // only a term without flips has five
+  }
+  __device__ __forceinline__ const float (&get() const)[5] { return s; }
+};
+template <> struct EnSign<double> {
+  uint32_t zz;
+  __device__ __forceinline__ EnSign(const EnTerm *, uint32_t code) : zz((code >> 8) & 15u) {}
+  __device__ __forceinline__ uint32_t get() const { return zz; }
+};
+// code bits 0-3: MC, bit 4: imaginary part, bit 5: E
+template <typename T, bool PAIR, typename C>
+__device__ __forceinline__ T en_pairs_rt(const C (&a)[EnAmp<T, PAIR>::N], uint32_t code, const EnSign<T> &sg) {
+  switch (code & (PAIR ? 63u : 31u)) {
+#define QW_PR(S) case S: return en_pairs<(S & 15), 0, (S >= 16), PAIR>(a, sg.get());
     QW_PR(0) QW_PR(1) QW_PR(2) QW_PR(3) QW_PR(4) QW_PR(5) QW_PR(6) QW_PR(7)
     QW_PR(8) QW_PR(9) QW_PR(10) QW_PR(11) QW_PR(12) QW_PR(13) QW_PR(14) QW_PR(15)
-    QW_PR(16) QW_PR(17) QW_PR(18) QW_PR(19) QW_PR(20) QW_PR(21) QW_PR(22) QW_PR(23)
+    QW_PR(17) QW_PR(18) QW_PR(19) QW_PR(20) QW_PR(21) QW_PR(22) QW_PR(23)
     QW_PR(24) QW_PR(25) QW_PR(26) QW_PR(27) QW_PR(28) QW_PR(29) QW_PR(30)
 #undef QW_PR
-    default: en_prod<T, TB, NC, 15, true>(q, a, v); break;
+    default: break;
   }
+  if constexpr (PAIR) {
+    switch (code & 63u) {
+#define QW_PR(S) case 32 + S: return en_pairs<(S & 15), 1, (S >= 16), PAIR>(a, sg.get());
+      QW_PR(0) QW_PR(1) QW_PR(2) QW_PR(3) QW_PR(4) QW_PR(5) QW_PR(6) QW_PR(7)
+      QW_PR(8) QW_PR(9) QW_PR(10) QW_PR(11) QW_PR(12) QW_PR(13) QW_PR(14) QW_PR(15)
+      QW_PR(16) QW_PR(17) QW_PR(18) QW_PR(19) QW_PR(20) QW_PR(21) QW_PR(22) QW_PR(23)
+      QW_PR(24) QW_PR(25) QW_PR(26) QW_PR(27) QW_PR(28) QW_PR(29) QW_PR(30) QW_PR(31)
+#undef QW_PR
+      default: break;
+    }
+  }
+  return en_pairs<15, 0, true, PAIR>(a, sg.get());
 }
 
-// Accumulates the terms [t0, t1) over the sub-block at `base` (a multiple of
-// 16 << TB) into acc, and the sub-block's squared norm into nrm.
-template <typename T, int TB, bool NC>
-__device__ __forceinline__ void energy_sub(const typename EnC<T>::t *__restrict__ psi, uint32_t dim,
-                                           const EnTerm *__restrict__ terms, uint32_t t0, uint32_t t1,
-                                           uint32_t base, typename AccOf<T>::t &acc, T &nrm) {
+template <typename T> __device__ __forceinline__ T en_coef(const uint4 &q);
+template <> __device__ __forceinline__ float en_coef<float>(const uint4 &q) { return __uint_as_float(q.z); }
+template <> __device__ __forceinline__ double en_coef<double>(const uint4 &q) {
+  return __hiloint2double((int)q.w, (int)q.z);
+}
+
+// Keeps the compiler from hoisting the pair products of every case of the
+// switch out of the term loop (they do not change in it, and their 240
+// values would be spilled).
+template <int N>
+__device__ __forceinline__ void en_pin(float2 (&a)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; k++) asm volatile("" : "+f"(a[k].x), "+f"(a[k].y));
+}
+template <int N>
+__device__ __forceinline__ void en_pin(double2 (&a)[N]) {
+#pragma unroll
+  for (int k = 0; k < N; k++) asm volatile("" : "+d"(a[k].x), "+d"(a[k].y));
+}
+
+// one term on the basis mask of combination MC
+template <typename T, int MC, bool PAIR, typename C>
+__device__ __forceinline__ void en_slot(const C (&a)[EnAmp<T, PAIR>::N], const EnTerm *t, uint32_t x0, T &e) {
+  const uint4 q = __ldg((const uint4 *)t);
+  const T coef = en_coef<T>(q);
+  const EnSign<T> sg(t, q.y);
+  const T c = (__popc(x0 & q.x) & 1) ? -coef : coef;
+  T s;
+  if constexpr (PAIR) {
+    if (q.y & 32u) {
+      if (q.y & 16u) s = en_pairs<MC, 1, true, PAIR>(a, sg.get());
+      else s = en_pairs<MC, 1, false, PAIR>(a, sg.get());
+      e = fma(c, s, e);
+      return;
+    }
+  }
+  if (q.y & 16u) s = en_pairs<MC, 0, true, PAIR>(a, sg.get());
+  else s = en_pairs<MC, 0, false, PAIR>(a, sg.get());
+  e = fma(c, s, e);
+}
+
+// Block `jb` of energy job J: 2^J.rep_bits coset representatives of each of
+// its class's groups, one per thread (blockDim.x = 2^J.rep_bits, at most
+// EN_THREADS), 2^J.iter_bits times; thread 0 writes {sum_k c_k term_k, squared norm
+// of the block} to out[0..1].  PAIR: FP32 states on a 16-byte boundary with a
+// layout built for pairs.
+template <typename T, bool PAIR, bool NC>
+__device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const EnTables &tab, double *out) {
   typedef typename EnC<T>::t C;
-  constexpr uint32_t JF = 15u << TB;  // the j-field of an index
-  const uint32_t own = base | threadIdx.x;
-  C a[16];
-#pragma unroll
-  for (int j = 0; j < 16; j++) {
-    const uint32_t x = own | ((uint32_t)j << TB);
-    if (x < dim) {
-      a[j] = en_ld<NC>(psi + x);
-    } else {
-      a[j].x = 0;
-      a[j].y = 0;
-    }
-    nrm += a[j].x * a[j].x + a[j].y * a[j].y;
-  }
-  const bool full = dim >= (16u << TB);
-  for (uint32_t t = t0; t < t1; t++) {
-    const uint2 w0 = __ldg((const uint2 *)&terms[t].xm);    // xm, zm
-    const uint2 w1 = __ldg((const uint2 *)&terms[t].skip);  // skip, flags
-    const T coef = (T)__ldg(&terms[t].coef);
-    const uint32_t xm = w0.x, zm = w0.y, skip = w1.x, fl = w1.y;
-    if (own & skip) continue;  // the pair is counted from its other member
-    const uint32_t ks = (skip & JF) >> TB;
-    const uint32_t mj = (xm & JF) >> TB, zj = (zm & JF) >> TB;
-    const uint32_t pb = own ^ (xm & ~JF);
-    const bool neg = __popc(own & zm) & 1;
-    T s = 0;
-    if (ks == 0 && full) {
-      T v[16];
-      en_prod_rt<T, TB, NC>(psi + pb, a, v, mj | (fl << 4));
-      s = en_signed16_bf<T>(v, zj);
-    } else {
-      // a skipped bit inside the j-field, or a register smaller than the
-      // sub-block: per-element tests
-#pragma unroll
-      for (int j = 0; j < 16; j++) {
-        const uint32_t x = own | ((uint32_t)j << TB);
-        if (((uint32_t)j & ks) || x >= dim) continue;
-        const C p = en_ld<NC>(psi + (pb | (((uint32_t)j ^ mj) << TB)));
-        const T v = fl ? (p.x * a[j].y - p.y * a[j].x) : (p.x * a[j].x + p.y * a[j].y);
-        s += (__popc((uint32_t)j & zj) & 1) ? -v : v;
-      }
-    }
-    acc.add(coef * (neg ? -s : s));
-  }
-}
-
-// Block `jb` (2^EN_BLOCK_BITS amplitudes) of energy job J, computed by a CTA
-// of THREADS threads in 4096 / (16 * THREADS) sub-blocks; thread 0 writes
-// {sum_k c_k term_k, squared norm of the block} to out[0..1].
-template <typename T, int THREADS, bool NC>
-__device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const EnClass *__restrict__ classes,
-                                             const EnTerm *__restrict__ terms, double *out) {
-  constexpr int TB = (THREADS == 256) ? 8 : 7;
-  constexpr int NSUB = (1 << EN_BLOCK_BITS) / (16 * THREADS);
-  static_assert((16 << TB) * NSUB == (1 << EN_BLOCK_BITS) && (1 << TB) == THREADS, "block shape");
+  constexpr int N = EnAmp<T, PAIR>::N;
   uint32_t c = J.class_begin;
   const uint32_t ce = J.class_begin + J.n_classes;
-  while (c + 1 < ce && classes[c + 1].block_begin <= jb) c++;
-  const EnClass K = classes[c];
-  const uint32_t within = jb - K.block_begin;
-  const uint32_t bpc_bits = (J.chunk_bits > (uint32_t)EN_BLOCK_BITS) ? J.chunk_bits - EN_BLOCK_BITS : 0u;
-  const uint32_t ownc = within >> bpc_bits;
-  const uint32_t bic = within & ((1u << bpc_bits) - 1u);
-  uint32_t chunk = ownc;
-  if (K.hb != 0xFFFFFFFFu) {  // own chunks are those with bit hb clear
-    const uint32_t p = K.hb - J.chunk_bits;
-    chunk = ((ownc >> p) << (p + 1)) | (ownc & ((1u << p) - 1u));
-  }
-  const uint32_t dim = 1u << J.n;
-  const uint32_t base = (chunk << J.chunk_bits) + (bic << EN_BLOCK_BITS);
-  typedef typename EnC<T>::t C;
+  while (c + 1 < ce && tab.classes[c + 1].block_begin <= jb) c++;
+  const EnClass K = tab.classes[c];
   const C *psi = (const C *)J.state;
   typename AccOf<T>::t acc;
   T nrm = 0;
+  const uint32_t n_rep = 1u << (J.n - EN_RANK - (PAIR ? 1 : 0));
 #pragma unroll 1
-  for (int sb = 0; sb < NSUB; sb++)
-    energy_sub<T, TB, NC>(psi, dim, terms, K.term_begin, K.term_end, base + ((uint32_t)sb << (TB + 4)), acc,
-                          nrm);
-  double e = acc.value();
-  double nn = (K.hb == 0xFFFFFFFFu) ? (double)nrm : 0.0;
-  __shared__ double en_red[2][THREADS / 32];
-  e = en_warp_sum(e);
-  nn = en_warp_sum(nn);
+  for (uint32_t it = 0; it < (1u << J.iter_bits); it++) {
+    const uint32_t j = ((((jb - K.block_begin) << J.iter_bits) + it) << J.rep_bits) | threadIdx.x;
+    if (j >= n_rep) break;
+#pragma unroll 1
+    for (uint32_t g = K.group_begin; g < K.group_end; g++) {
+      const uint4 b = __ldg((const uint4 *)(tab.groups + g)), w = __ldg((const uint4 *)(tab.groups + g) + 1);
+      const uint32_t basis[EN_RANK] = {b.x, b.y, b.z, b.w};
+      // zeros at the pivots, ascending (and at bit 0 of a pair)
+      uint32_t x = PAIR ? j << 1 : j;
+#pragma unroll
+      for (int k = 0; k < EN_RANK; k++) {
+        const uint32_t lo = x & ((1u << ((w.x >> (8 * k)) & 31u)) - 1u);
+        x = ((x ^ lo) << 1) | lo;
+      }
+      const uint32_t x0 = x;
+      C a[N];
+#pragma unroll
+      for (int k = 0; k < 16; k++) {  // Gray-code order, one XOR per address
+        if (k) x ^= basis[(k & 1) ? 0 : (k & 2) ? 1 : (k & 4) ? 2 : 3];
+        const int i = k ^ (k >> 1);
+        if constexpr (PAIR) {
+          const float4 v = en_ld<NC>((const float4 *)(psi + x));
+          a[2 * i] = make_float2(v.x, v.y);
+          a[2 * i + 1] = make_float2(v.z, v.w);
+        } else {
+          a[i] = en_ld<NC>(psi + x);
+        }
+      }
+      if (w.w & EN_GROUP_NORM) {
+        T s = 0;
+#pragma unroll
+        for (int k = 0; k < N; k++) s += a[k].x * a[k].x + a[k].y * a[k].y;
+        nrm += s;
+      }
+      T e = 0;
+      uint32_t t = w.y;
+      // the first terms flip the basis masks, one each: straight-line code, a
+      // uniform branch or two each (random Hamiltonians hold few others)
+      const uint32_t ns = w.w >> EN_GROUP_SLOTS_SHIFT;
+      if (ns > 0) en_slot<T, 1, PAIR>(a, tab.terms + t, x0, e);
+      if (ns > 1) en_slot<T, 2, PAIR>(a, tab.terms + t + 1, x0, e);
+      if (ns > 2) en_slot<T, 4, PAIR>(a, tab.terms + t + 2, x0, e);
+      if (ns > 3) en_slot<T, 8, PAIR>(a, tab.terms + t + 3, x0, e);
+      t += ns;
+#pragma unroll 1
+      for (uint32_t i = 0; t < w.z; t++, i++) {
+        if ((i & 3u) == 0) {  // at most four terms between two-sums
+          acc.add(e);
+          e = 0;
+        }
+        const uint4 q = __ldg((const uint4 *)(tab.terms + t));  // zm, code, coef
+        const T coef = en_coef<T>(q);
+        const EnSign<T> sg(tab.terms + t, q.y);
+        en_pin(a);
+        const T s = en_pairs_rt<T, PAIR>(a, q.y, sg);
+        e = fma((__popc(x0 & q.x) & 1) ? -coef : coef, s, e);
+      }
+      acc.add(e);
+    }
+  }
+  __shared__ double en_red[2][8];
+  const double e = en_warp_total(acc), nn = en_warp_total_norm(nrm);
   const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
   if (ln == 0) { en_red[0][w] = e; en_red[1][w] = nn; }
   __syncthreads();
   if (threadIdx.x == 0) {
     double se = 0, sn = 0;
-    for (int i = 0; i < THREADS / 32; i++) { se += en_red[0][i]; sn += en_red[1][i]; }
+    for (uint32_t i = 0; i < blockDim.x / 32; i++) { se += en_red[0][i]; sn += en_red[1][i]; }
     out[0] = se;
     out[1] = sn;
   }

@@ -412,6 +412,7 @@ struct DeviceState {
   std::vector<void *> task_state;  // state a task's observables read
   std::vector<Wave> waves;
   EnClass *d_classes = nullptr;
+  EnGroup *d_groups = nullptr;
   EnTerm *d_terms = nullptr;
   std::vector<uint32_t> ham_class_off;
   double *d_partials = nullptr;
@@ -797,18 +798,25 @@ static void prepare(qw_plan *P) {
 
   // Hamiltonians
   std::vector<EnClass> cls;
+  std::vector<EnGroup> grp;
   std::vector<EnTerm> trm;
   for (auto &H : P->hams) {
     D->ham_class_off.push_back((uint32_t)cls.size());
-    const uint32_t toff = (uint32_t)trm.size();
-    for (EnClass c : H.classes) {
-      c.term_begin += toff;
-      c.term_end += toff;
+    const uint32_t goff = (uint32_t)grp.size(), toff = (uint32_t)trm.size();
+    for (EnClass c : H.en.classes) {
+      c.group_begin += goff;
+      c.group_end += goff;
       cls.push_back(c);
     }
-    trm.insert(trm.end(), H.terms.begin(), H.terms.end());
+    for (EnGroup g : H.en.groups) {
+      g.term_begin += toff;
+      g.term_end += toff;
+      grp.push_back(g);
+    }
+    trm.insert(trm.end(), H.en.terms.begin(), H.en.terms.end());
   }
   D->d_classes = D->arena.upload(cls, s);
+  D->d_groups = D->arena.upload(grp, s);
   D->d_terms = D->arena.upload(trm, s);
 
   // results
@@ -979,12 +987,13 @@ static void prepare(qw_plan *P) {
         j.state = D->task_state[t];
         j.out = D->d_energy + 2 * (size_t)t;
         j.n = H.n_eff;
-        j.chunk_bits = H.chunk_bits;
+        j.rep_bits = H.en.rep_bits;
+        j.iter_bits = H.en.iter_bits;
         j.class_begin = D->ham_class_off[tp.ham];
-        j.n_classes = (uint32_t)H.classes.size();
+        j.n_classes = (uint32_t)H.en.classes.size();
         j.block_begin = W.en_blocks;
-        j.n_blocks = H.n_blocks;
-        W.en_blocks += H.n_blocks;
+        j.n_blocks = H.en.n_blocks;
+        W.en_blocks += H.en.n_blocks;
         W.en.push_back(j);
         W.obs_tasks_en.push_back(t);
       }
@@ -1032,19 +1041,15 @@ static void prepare(qw_plan *P) {
         const EnJob &j = W.en[e];
         const double Sj = (double)sv_state_bytes(fp64, j.n);
         P->energy_alg_bytes += (double)j.n_classes * Sj;
-        // L2 -> SM reads: own amplitudes once per class, and half the state
-        // per flipping term (each pair is read from one side)
-        const HamLayout &H = P->hams[P->tasks[W.obs_tasks_en[e]].ham];
-        size_t flipping = 0;
-        for (const EnTerm &t : H.terms) flipping += (t.xm != 0);
-        P->energy_l2_bytes += (double)j.n_classes * Sj + 0.5 * Sj * (double)flipping;
+        // L2 -> SM reads: the state once per group of terms
+        P->energy_l2_bytes += (double)P->hams[P->tasks[W.obs_tasks_en[e]].ham].en.groups.size() * Sj;
       }
       // persistent work list: pass jobs, then (fused) the energy jobs,
       // released in the order their states finish
       std::vector<SvJob> up = W.jobs;
-      W.grid = !W.per_pass ? sv_batch_grid(fp64, W.k_max, E->sm_count, W.ar) : 0;
       W.fused_energy =
           !W.per_pass && P->opts.fuse_energy && !W.en.empty() && sv_threads_for_k(W.k_max, W.ar, fp64) == 128;
+      W.grid = !W.per_pass ? sv_batch_grid(fp64, W.k_max, E->sm_count, W.ar, W.fused_energy) : 0;
       if (W.fused_energy) {
         std::vector<SvJob> ej;
         for (size_t e = 0; e < W.en.size(); e++) {
@@ -1361,7 +1366,8 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
     if (!W.per_pass) {
       if (W.total_items) {
         CK(cudaMemsetAsync(W.d_ctr, 0, W.ctr_words * sizeof(unsigned int), s));
-        EnTables et{W.d_en, D->d_classes, D->d_terms, D->d_partials};
+        const EnTables et =
+            W.fused_energy ? EnTables{W.d_en, D->d_classes, D->d_groups, D->d_terms, D->d_partials} : EnTables{};
         launch_sv_batch(W.fp64, T, W.d_jobs, W.d_segs, W.seg_bits, W.total_items, W.k_max, W.d_ctr, et,
                         W.grid, s, W.ar);
         nl += 1;
@@ -1381,8 +1387,8 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
       launch_energy_reduce(W.d_en, (uint32_t)W.en.size(), D->d_partials, s);
       nl += 1;
     } else {
-      launch_energy(W.fp64, W.d_en, (uint32_t)W.en.size(), W.en_blocks, D->d_classes, D->d_terms,
-                    D->d_partials, s);
+      const EnTables et{W.d_en, D->d_classes, D->d_groups, D->d_terms, D->d_partials};
+      launch_energy(W.fp64, !W.fp64, et, (uint32_t)W.en.size(), W.en_blocks, W.en.empty() ? 0u : W.en[0].rep_bits, s);
       if (!W.en.empty()) nl += 2;
     }
     if (!W.src.empty()) nl += W.shots.empty() ? 2 : 3;
@@ -2123,9 +2129,10 @@ qw_status sv_energy_dev(Engine *E, uint32_t mode, uint32_t n, const void *state,
   CK(cudaSetDevice(E->device));
   cudaStream_t s = (cudaStream_t)stream;
   const bool fp64 = mode == QW_MODE_SV_FP64;
-  HamLayout H;
-  build_energy_layout(terms, n_terms, n, fp64 ? 16u : 8u, &H.chunk_bits, H.classes, H.terms, &H.n_blocks);
+  const bool pair = en_pair(fp64, state);
+  const EnLayout H = build_energy_layout(terms, n_terms, n, fp64, pair, en_rep_bits(n));
   EnClass *dc = stream_upload(H.classes, s);
+  EnGroup *dg = stream_upload(H.groups, s);
   EnTerm *dt = stream_upload(H.terms, s);
   double *dout = nullptr, *dpart = nullptr;
   CK(cudaMallocAsync((void **)&dout, 2 * sizeof(double), s));
@@ -2134,16 +2141,18 @@ qw_status sv_energy_dev(Engine *E, uint32_t mode, uint32_t n, const void *state,
   j.state = state;
   j.out = dout;
   j.n = n;
-  j.chunk_bits = H.chunk_bits;
+  j.rep_bits = H.rep_bits;
+  j.iter_bits = H.iter_bits;
   j.class_begin = 0;
   j.n_classes = (uint32_t)H.classes.size();
   j.block_begin = 0;
   j.n_blocks = H.n_blocks;
   EnJob *dj = stream_upload(std::vector<EnJob>{j}, s);
-  launch_energy(fp64, dj, 1, H.n_blocks, dc, dt, dpart, s);
+  launch_energy(fp64, pair, EnTables{dj, dc, dg, dt, dpart}, 1, H.n_blocks, H.rep_bits, s);
   double res[2];
   CK(cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, s));
   CK(cudaFreeAsync(dc, s));
+  CK(cudaFreeAsync(dg, s));
   CK(cudaFreeAsync(dt, s));
   CK(cudaFreeAsync(dout, s));
   CK(cudaFreeAsync(dpart, s));

@@ -12,8 +12,10 @@
 // loads this library holds until the process exits.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstddef>
 #include <mutex>
+#include <new>
 
 #include "qw_internal.h"
 
@@ -21,14 +23,19 @@ namespace qw {
 
 namespace {
 
-constexpr uint32_t NA_MAX_CLASSES = 8;
-// blocks of the largest register: 2^u class-0 chunks plus 2^(u-1) chunks
-// for each other class, times the blocks per chunk (u = 3 above 15 qubits)
-constexpr uint32_t NA_MAX_BLOCKS = (1u << (QW_NOALLOC_MAX_QUBITS - 3 - EN_BLOCK_BITS)) * (8u + 7u * 4u);
+constexpr uint32_t NA_CLASS_BITS = 3, NA_MAX_CLASSES = 1u << NA_CLASS_BITS;
+// every group of a class but its last holds EN_RANK independent masks, so at
+// least as many terms
+constexpr uint32_t NA_MAX_GROUPS = QW_NOALLOC_MAX_TERMS / EN_RANK + NA_MAX_CLASSES + 1;
+// blocks of the largest register
+constexpr uint32_t NA_REP_BITS = en_rep_bits(QW_NOALLOC_MAX_QUBITS);
+constexpr uint32_t NA_MAX_BLOCKS = NA_MAX_CLASSES << (QW_NOALLOC_MAX_QUBITS - EN_RANK - NA_REP_BITS -
+                                                      en_iter_bits(QW_NOALLOC_MAX_QUBITS, NA_REP_BITS));
 
-struct NaHeader {
-  EnJob job;
-  EnClass classes[NA_MAX_CLASSES];
+struct alignas(16) NaHeader {
+  alignas(16) EnJob job;
+  alignas(16) EnClass classes[NA_MAX_CLASSES];
+  EnGroup groups[NA_MAX_GROUPS];
   EnTerm terms[QW_NOALLOC_MAX_TERMS];
 };
 struct NaScratch {
@@ -38,7 +45,7 @@ struct NaScratch {
 
 }  // namespace
 
-// The scratch array (about 1.2 MB).  In host code this name is only a
+// The scratch array (about 1.1 MB).  In host code this name is only a
 // stand-in for the device object: its device address comes from
 // cudaGetSymbolAddress.
 static __device__ __align__(256) unsigned char qw_noalloc_scratch[sizeof(NaScratch)];
@@ -67,66 +74,15 @@ qw_status scratch_address(int dev, NaScratch **out) {
   return QW_OK;
 }
 
-// Term layout for the fixed arrays: classes by the flip bits above the
-// chunk, term order kept inside a class, as in the allocating entry point,
-// but always with 3 class bits once n >= 15 (chunks of an eighth of the
-// state), so that every layout fits NA_MAX_CLASSES and NA_MAX_BLOCKS.  The
-// allocating entry point sizes chunks to at most EN_CHUNK_BYTES instead
-// (one class for FP32 states up to 22 qubits, chunks of 64 MB at 26): the
-// two compute the same terms with the same kernel, adding them in a
-// different order and at a different speed.
-void layout_fixed(const qw_pauli_term *terms, uint32_t n_terms, uint32_t n, NaHeader &h,
-                  uint32_t *n_classes, uint32_t *n_blocks, uint32_t *chunk_bits_out) {
-  uint32_t u = 0, chunk_bits = n;
-  if (n >= (uint32_t)EN_BLOCK_BITS) {
-    u = (n - EN_BLOCK_BITS < 3u) ? n - EN_BLOCK_BITS : 3u;
-    chunk_bits = n - u;
-  }
-  const uint32_t bpc = (chunk_bits >= (uint32_t)EN_BLOCK_BITS) ? (1u << (chunk_bits - EN_BLOCK_BITS)) : 1u;
-  uint32_t count[NA_MAX_CLASSES] = {0}, start[NA_MAX_CLASSES] = {0};
-  for (uint32_t k = 0; k < n_terms; k++) count[(uint32_t)(terms[k].xmask >> chunk_bits)]++;
-  uint32_t nc = 0, blk = 0, off = 0;
-  for (uint32_t d = 0; d < (1u << u); d++) {
-    if (d != 0 && count[d] == 0) continue;
-    EnClass c{};
-    c.term_begin = off;
-    c.term_end = off + count[d];
-    c.hb = (d == 0) ? 0xFFFFFFFFu : (chunk_bits + 31 - __builtin_clz(d));
-    c.n_own = (d == 0) ? (1u << u) : (1u << (u - 1));
-    c.block_begin = blk;
-    blk += c.n_own * bpc;
-    start[d] = off;
-    off += count[d];
-    h.classes[nc++] = c;
-  }
-  uint32_t fill[NA_MAX_CLASSES] = {0};
-  for (uint32_t k = 0; k < n_terms; k++) {
-    const uint64_t m = terms[k].xmask, z = terms[k].zmask;
-    const int y = __builtin_popcountll(m & z);
-    const double sgn = ((y & 3) == 0 || (y & 3) == 3) ? 1.0 : -1.0;
-    const uint32_t d = (uint32_t)(m >> chunk_bits);
-    EnTerm t{};
-    t.xm = (uint32_t)m;
-    t.zm = (uint32_t)z;
-    t.flags = (uint32_t)(y & 1);
-    t.coef = terms[k].coef * sgn * (m ? 2.0 : 1.0);
-    t.skip = (d == 0 && m != 0) ? (1u << (63 - __builtin_clzll(m))) : 0u;
-    h.terms[start[d] + fill[d]++] = t;
-  }
-  *n_classes = nc;
-  *n_blocks = blk;
-  *chunk_bits_out = chunk_bits;
+// Copies a piece of the host-built layout, passed by value as the kernel's
+// parameter (the device reads no host memory), into the scratch array.
+struct NaPiece {
+  uint4 w[1024];
+};
+static_assert(sizeof(NaPiece) <= 32000 && sizeof(NaHeader) % 16 == 0, "pieces fit the kernel parameter space");
+__global__ void na_setup_kernel(const NaPiece h, uint4 *dst, uint32_t n) {
+  for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) dst[i] = h.w[i];
 }
-
-// Copies the host-built layout, passed by value as the kernel's parameter
-// (the device reads no host memory), into the scratch array.
-__global__ void na_setup_kernel(const NaHeader h, NaHeader *dst, uint32_t words) {
-  const uint32_t *src = (const uint32_t *)&h;
-  uint32_t *d = (uint32_t *)dst;
-  for (uint32_t i = threadIdx.x; i < words; i += blockDim.x) d[i] = src[i];
-}
-static_assert(sizeof(NaHeader) <= 32000, "layout must fit the kernel parameter space");
-static_assert(sizeof(NaHeader) % 4 == 0, "layout is copied in 32-bit words");
 
 }  // namespace
 }  // namespace qw
@@ -173,33 +129,58 @@ extern "C" qw_status qw_sv_energy_noalloc_dev(uint32_t mode, uint32_t n, const v
   qw_status st = scratch_address(dev, &S);
   if (st != QW_OK) return st;
 
+  // The term layout of the allocating entry point with at most 3 class bits,
+  // so that it fits the fixed arrays (chunks of an eighth of the state above
+  // 25 qubits, where the allocating one takes smaller ones: the same terms,
+  // added in another order)
+  const bool fp64 = mode == QW_MODE_SV_FP64, pair = en_pair(fp64, state);
   NaHeader h;  // built on the host stack, handed to the device as a kernel parameter
-  uint32_t n_classes = 0, n_blocks = 0, chunk_bits = 0;
-  layout_fixed(terms, (uint32_t)n_terms, n, h, &n_classes, &n_blocks, &chunk_bits);
-  h.job.state = state;
-  h.job.out = out;
-  h.job.n = n;
-  h.job.chunk_bits = chunk_bits;
-  h.job.class_begin = 0;
-  h.job.n_classes = n_classes;
-  h.job.block_begin = 0;
-  h.job.n_blocks = n_blocks;
+  uint32_t n_blocks = 0;
+  try {
+    const EnLayout L = build_energy_layout(terms, n_terms, n, fp64, pair, en_rep_bits(n), NA_CLASS_BITS);
+    if (L.classes.size() > NA_MAX_CLASSES || L.groups.size() > NA_MAX_GROUPS || L.n_blocks > NA_MAX_BLOCKS) {
+      set_last_error("the term layout exceeds the scratch array");
+      return QW_ERR_BUDGET;
+    }
+    std::copy(L.classes.begin(), L.classes.end(), h.classes);
+    std::copy(L.groups.begin(), L.groups.end(), h.groups);
+    std::copy(L.terms.begin(), L.terms.end(), h.terms);
+    h.job.state = state;
+    h.job.out = out;
+    h.job.n = n;
+    h.job.rep_bits = L.rep_bits;
+    h.job.iter_bits = L.iter_bits;
+    h.job.class_begin = 0;
+    h.job.n_classes = (uint32_t)L.classes.size();
+    h.job.block_begin = 0;
+    h.job.n_blocks = n_blocks = L.n_blocks;
+  } catch (const std::bad_alloc &) {
+    set_last_error("host allocation failed");
+    return QW_ERR_OOM;
+  }
   // every partial is written by its block before the reduction reads it, so
   // nothing in the array needs clearing between calls
   cudaStream_t s = (cudaStream_t)stream;
   char *base = (char *)S;  // device address: offsets only, never dereferenced here
   EnJob *d_job = (EnJob *)(base + offsetof(NaScratch, h) + offsetof(NaHeader, job));
   EnClass *d_classes = (EnClass *)(base + offsetof(NaScratch, h) + offsetof(NaHeader, classes));
+  EnGroup *d_groups = (EnGroup *)(base + offsetof(NaScratch, h) + offsetof(NaHeader, groups));
   EnTerm *d_terms = (EnTerm *)(base + offsetof(NaScratch, h) + offsetof(NaHeader, terms));
   double *d_partials = (double *)(base + offsetof(NaScratch, partials));
   const size_t hdr = offsetof(NaHeader, terms) + sizeof(EnTerm) * (size_t)n_terms;
-  na_setup_kernel<<<1, 256, 0, s>>>(h, (NaHeader *)(base + offsetof(NaScratch, h)), (uint32_t)(hdr / 4));
+  for (size_t o = 0; o < hdr; o += sizeof(NaPiece)) {
+    NaPiece piece;
+    const size_t k = std::min(sizeof(NaPiece), hdr - o);
+    memcpy(&piece, (const char *)&h + o, k);
+    na_setup_kernel<<<1, 256, 0, s>>>(piece, (uint4 *)(base + offsetof(NaScratch, h) + o), (uint32_t)(k / 16));
+  }
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_error(std::string("layout copy failed: ") + cudaGetErrorString(e));
     return QW_ERR_CUDA;
   }
-  launch_energy(mode == QW_MODE_SV_FP64, d_job, 1, n_blocks, d_classes, d_terms, d_partials, s);
+  launch_energy(fp64, pair, EnTables{d_job, d_classes, d_groups, d_terms, d_partials}, 1, n_blocks,
+                en_rep_bits(n), s);
   e = cudaGetLastError();
   if (e != cudaSuccess) {
     set_last_error(std::string("energy launch failed: ") + cudaGetErrorString(e));

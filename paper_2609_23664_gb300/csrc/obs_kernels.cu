@@ -2,13 +2,10 @@
 //
 // Energy (the repeated expectation evaluation of the VQE workloads, Sec. V,
 // Table III): E = sum_k c_k <psi|P_k|psi> / <psi|psi> with
-// P|x> = i^{#Y} (-1)^{popc(x&z)} |x^m>.  For m != 0 the pair (x, x^m) is
-// visited once from the side whose highest flipped bit is 0, contributing
-// 2 Re(i^{#Y} (-1)^{popc(x&z)} conj(psi[x^m]) psi[x]).  Terms are grouped by
-// the flipped bits above an L2-sized chunk, so that all terms of a class touch
-// only one pair of chunks and the pair stays L2-resident while the class runs.
-// Products are FP32; every thread keeps a double-float (two-sum) accumulator
-// across terms, and block and final reductions are FP64, in a fixed order.
+// P|x> = i^{#Y} (-1)^{popc(x&z)} |x^m>, evaluated in groups of terms on the
+// cosets of their flip masks (energy_block.cuh).  Products are FP32; every
+// thread keeps a double-float (two-sum) accumulator across groups, and block
+// and final reductions are FP64, in a fixed order.
 //
 // Sampling: p_x = |psi_x|^2 summed in FP64 into a CDF that is never written
 // out: per 4096-amplitude block a lane sums 128 contiguous probabilities and
@@ -19,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <unordered_map>
 
 #include "energy_block.cuh"
 #include "qw_internal.h"
@@ -32,88 +30,185 @@ template <> struct V2o<double> { typedef double2 t; };
 // ---------------------------------------------------------------------------
 // energy layout (host)
 // ---------------------------------------------------------------------------
-void build_energy_layout(const qw_pauli_term *terms, uint64_t n_terms, uint32_t n, uint32_t amp_bytes,
-                         uint32_t *chunk_bits_out, std::vector<EnClass> &classes,
-                         std::vector<EnTerm> &en_terms, uint32_t *n_blocks) {
+EnLayout build_energy_layout(const qw_pauli_term *terms, uint64_t n_terms, uint32_t n, bool fp64, bool pair,
+                             uint32_t rep_bits, uint32_t max_class_bits) {
+  const uint32_t amp_bytes = fp64 ? 16u : 8u;
+  const uint32_t low = pair ? 1u : 0u;  // bit 0 is a direction of every pair layout's cosets
+  EnLayout L;
+  L.rep_bits = rep_bits;
   // chunks of at most EN_CHUNK_BYTES, so that the chunk pair a class reads
-  // stays in L2 (a quarter of the state as the chunk measured fastest for
-  // 24 FP32 qubits on GB300: 186 ms against 202 ms with an eighth, 188 ms
-  // with a half, 247 ms with a sixteenth), and no smaller than a block
+  // stays in L2, and large enough for a coset's in-chunk pivots
   uint32_t chunk_bits = n;
-  while (chunk_bits > (uint32_t)EN_BLOCK_BITS && ((uint64_t)amp_bytes << chunk_bits) > EN_CHUNK_BYTES) chunk_bits--;
+  while (chunk_bits > (uint32_t)(EN_RANK + 8) && n - chunk_bits < max_class_bits &&
+         ((uint64_t)amp_bytes << chunk_bits) > EN_CHUNK_BYTES)
+    chunk_bits--;
   const uint32_t u = n - chunk_bits;
-  const uint32_t bpc = (chunk_bits >= (uint32_t)EN_BLOCK_BITS) ? (1u << (chunk_bits - EN_BLOCK_BITS)) : 1u;
-  std::vector<std::vector<EnTerm>> by_class(1u << u);
+  // per class: distinct masks (but for a pair's bit 0) in order of appearance, each with its terms
+  struct Flip {
+    uint32_t mask;
+    std::vector<uint64_t> terms;
+    bool used = false;
+  };
+  std::vector<std::vector<Flip>> by_class(1u << u);
+  std::vector<std::unordered_map<uint32_t, size_t>> at(1u << u);
   for (uint64_t k = 0; k < n_terms; k++) {
-    const uint64_t m = terms[k].xmask, z = terms[k].zmask;
-    const int y = __builtin_popcountll(m & z);
-    const double sgn = ((y & 3) == 0 || (y & 3) == 3) ? 1.0 : -1.0;
-    EnTerm t{};
-    t.xm = (uint32_t)m;
-    t.zm = (uint32_t)z;
-    t.flags = (uint32_t)(y & 1);
-    t.coef = terms[k].coef * sgn * (m ? 2.0 : 1.0);
-    const uint32_t d = (uint32_t)(m >> chunk_bits);
-    t.skip = (d == 0 && m != 0) ? (1u << (63 - __builtin_clzll(m))) : 0u;
-    by_class[d].push_back(t);
+    const uint32_t m = (uint32_t)terms[k].xmask & ~low, d = (uint32_t)((uint64_t)m >> chunk_bits);
+    auto it = at[d].emplace(m, by_class[d].size());
+    if (it.second) by_class[d].push_back(Flip{m, {}});
+    by_class[d][it.first->second].terms.push_back(k);
   }
-  classes.clear();
-  en_terms.clear();
+  L.iter_bits = en_iter_bits(n, rep_bits);
+  const uint32_t reps = n - EN_RANK - low;
+  const uint32_t blocks = reps > rep_bits + L.iter_bits ? 1u << (reps - rep_bits - L.iter_bits) : 1u;
   uint32_t blk = 0;
   for (uint32_t d = 0; d < (1u << u); d++) {
-    if (d != 0 && by_class[d].empty()) continue;
+    std::vector<Flip> &F = by_class[d];
+    if (d != 0 && F.empty()) continue;
     EnClass c{};
-    c.term_begin = (uint32_t)en_terms.size();
-    en_terms.insert(en_terms.end(), by_class[d].begin(), by_class[d].end());
-    c.term_end = (uint32_t)en_terms.size();
-    c.hb = (d == 0) ? 0xFFFFFFFFu : (chunk_bits + 31 - __builtin_clz(d));
-    c.n_own = (d == 0) ? (1u << u) : (1u << (u - 1));
+    c.group_begin = (uint32_t)L.groups.size();
+    size_t next = 0;
+    bool first = true;
+    for (;;) {
+      while (next < F.size() && F[next].used) next++;
+      if (next == F.size() && !(d == 0 && first)) break;
+      EnGroup g{};
+      uint32_t ech[EN_RANK] = {0}, rank = 0;  // echelon form of the basis (distinct leading bits)
+      auto reduce = [&](uint32_t v) {
+        for (uint32_t i = 0; i < rank; i++) v = std::min(v, v ^ ech[i]);
+        return v;
+      };
+      auto push = [&](uint32_t v) {
+        const uint32_t r = reduce(v);
+        if (!r) return false;
+        g.basis[rank] = v;
+        // kept descending, so that reducing in order clears leading bits once
+        uint32_t i = rank++;
+        for (; i > 0 && ech[i - 1] < r; i--) ech[i] = ech[i - 1];
+        ech[i] = r;
+        return true;
+      };
+      for (size_t i = next; i < F.size() && rank < (uint32_t)EN_RANK; i++)
+        if (!F[i].used && F[i].mask) push(F[i].mask);
+      // fewer masks than EN_RANK: unit vectors, from bit 5 up so that a
+      // warp's representatives stay consecutive
+      for (uint32_t i = 0; i < chunk_bits && rank < (uint32_t)EN_RANK; i++)
+        push((1u << ((i + 5) % chunk_bits)) & ~low);
+      uint32_t piv[EN_RANK];
+      for (uint32_t i = 0; i < (uint32_t)EN_RANK; i++) piv[i] = 31u - (uint32_t)__builtin_clz(ech[EN_RANK - 1 - i]);
+      for (uint32_t i = 0; i < (uint32_t)EN_RANK; i++) g.pivots |= piv[i] << (8 * i);
+      if (d == 0 && first) g.flags |= EN_GROUP_NORM;
+      // every term whose mask lies in the span
+      g.term_begin = (uint32_t)L.terms.size();
+      auto put = [&](uint64_t k, uint32_t comb) {
+        const uint64_t m = terms[k].xmask, z = terms[k].zmask;
+        const int y = __builtin_popcountll(m & z);
+        EnTerm t{};
+        t.zm = (uint32_t)z;
+        t.code = comb | ((uint32_t)(y & 1) << 4);
+        if (m & low) t.code |= 32u;
+        float sg[EN_RANK + 1];
+        uint32_t ns = 0;
+        // the highest flipped direction has no sign: a basis vector, bit 0
+        // of a pair, or none
+        const int top = comb ? 31 - __builtin_clz(comb) : ((m & low) ? -1 : EN_RANK);
+        if (pair && top != -1) sg[ns++] = (z & 1u) ? -1.f : 1.f;
+        for (int i = 0; i < EN_RANK; i++) {
+          const uint32_t par = (uint32_t)(__builtin_popcountll(g.basis[i] & z) & 1);
+          t.code |= par << (8 + i);
+          if (i != top) sg[ns++] = par ? -1.f : 1.f;
+        }
+        if (ns == EN_RANK + 1 && sg[EN_RANK] < 0) t.code |= EN_LAST_SIGN;
+        for (uint32_t i = 0; i < std::min<uint32_t>(ns, EN_RANK); i++) t.sign[i] = sg[i];
+        const double coef = terms[k].coef * (((y & 3) == 0 || (y & 3) == 3) ? 1.0 : -1.0) * (m ? 2.0 : 1.0);
+        if (amp_bytes == 16) t.coef64 = coef;
+        else t.coef32 = (float)coef;
+        L.terms.push_back(t);
+      };
+      auto flip_of = [&](uint32_t comb) -> Flip * {
+        uint32_t m = 0;
+        for (uint32_t i = 0; i < (uint32_t)EN_RANK; i++)
+          if ((comb >> i) & 1u) m ^= g.basis[i];
+        auto it = at[d].find(m);
+        return (it == at[d].end() || F[it->second].used) ? nullptr : &F[it->second];
+      };
+      // one term of each basis mask that is a term's mask (the first ones of
+      // the basis) first
+      uint32_t slots = 0;
+      while (slots < (uint32_t)EN_RANK) {
+        const Flip *f = flip_of(1u << slots);
+        if (!f) break;
+        put(f->terms[0], 1u << slots++);
+      }
+      g.flags |= slots << EN_GROUP_SLOTS_SHIFT;
+      for (uint32_t comb = (d == 0 && first) ? 0u : 1u; comb < (1u << EN_RANK); comb++) {
+        Flip *f = flip_of(comb);
+        if (!f) continue;
+        f->used = true;
+        const bool slotted = comb && (comb & (comb - 1)) == 0 && comb < (1u << slots);
+        for (size_t i = slotted ? 1 : 0; i < f->terms.size(); i++) put(f->terms[i], comb);
+      }
+      g.term_end = (uint32_t)L.terms.size();
+      L.groups.push_back(g);
+      first = false;
+    }
+    c.group_end = (uint32_t)L.groups.size();
     c.block_begin = blk;
-    blk += c.n_own * bpc;
-    classes.push_back(c);
+    blk += blocks;
+    L.classes.push_back(c);
   }
-  *chunk_bits_out = chunk_bits;
-  *n_blocks = blk;
+  L.n_blocks = blk;
+  return L;
 }
 
 // ---------------------------------------------------------------------------
 // energy kernels
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double warp_sum_d(double v) { return en_warp_sum(v); }
-
-// one CTA per 4096-amplitude block; the block's job is found by binary search.
-// Four CTAs per SM (64 registers for FP32): the kernel is bound by the
-// latency and bandwidth of its L2 partner reads, so resident warps matter
-// more than registers.
-template <typename T>
-__global__ void __launch_bounds__(EN_THREADS, 4)
-energy_kernel(const EnJob *__restrict__ jobs, uint32_t n_jobs, const EnClass *__restrict__ classes,
-              const EnTerm *__restrict__ terms, double *partials) {
+// one CTA per block; the block's job is found by binary search.  The 64
+// registers of an FP32 pair coset leave five CTAs of 128 threads per SM (96
+// registers): 64 24-qubit states, 200 terms: 27.7 ms, against 30.9 ms with
+// four CTAs, 33.6 ms with six (which spill), 31.6 ms with two of 256 threads,
+// 33.1 ms for cosets of 16 amplitudes on 32 warps per SM (bound by
+// instruction issue) and 47 ms term by term.
+template <typename T, bool PAIR>
+__global__ void __launch_bounds__(EN_THREADS, sizeof(T) == 8 ? 4 : PAIR ? 5 : 8)
+energy_kernel(EnTables t, uint32_t n_jobs) {
   const uint32_t gb = blockIdx.x;
   uint32_t lo = 0, hi = n_jobs;
   while (hi - lo > 1) {
     const uint32_t mid = (lo + hi) >> 1;
-    if (jobs[mid].block_begin <= gb) lo = mid; else hi = mid;
+    if (t.jobs[mid].block_begin <= gb) lo = mid; else hi = mid;
   }
-  const EnJob J = jobs[lo];
-  energy_block<T, EN_THREADS, true>(J, gb - J.block_begin, classes, terms, partials + 2 * (size_t)gb);
+  const EnJob J = t.jobs[lo];
+  energy_block<T, PAIR, true>(J, gb - J.block_begin, t, t.partials + 2 * (size_t)gb);
 }
 
-// one warp per job; fixed summation order
-__global__ void energy_reduce_kernel(const EnJob *__restrict__ jobs, uint32_t n_jobs,
-                                     const double *__restrict__ partials) {
-  const uint32_t j = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-  const int ln = threadIdx.x & 31;
-  if (j >= n_jobs) return;
-  const EnJob J = jobs[j];
+// one CTA per job; fixed summation order.  (One warp per job took 2.2 ms for
+// the 262144 partials of a 26-qubit state, as long as the energy kernel.)
+constexpr int EN_RED_THREADS = 256;
+__global__ void __launch_bounds__(EN_RED_THREADS)
+energy_reduce_kernel(const EnJob *__restrict__ jobs, const double2 *__restrict__ partials) {
+  const EnJob J = jobs[blockIdx.x];
   double se = 0, sn = 0;
-  for (uint32_t i = ln; i < J.n_blocks; i += 32) {
-    se += partials[2 * (size_t)(J.block_begin + i)];
-    sn += partials[2 * (size_t)(J.block_begin + i) + 1];
+#pragma unroll 8
+  for (uint32_t i = threadIdx.x; i < J.n_blocks; i += EN_RED_THREADS) {
+    const double2 v = partials[J.block_begin + i];
+    se += v.x;
+    sn += v.y;
   }
-  se = warp_sum_d(se);
-  sn = warp_sum_d(sn);
-  if (ln == 0) {
+  __shared__ double red[2][EN_RED_THREADS / 32];
+  se = en_warp_sum(se);
+  sn = en_warp_sum(sn);
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = se;
+    red[1][threadIdx.x >> 5] = sn;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    se = sn = 0;
+    for (int i = 0; i < EN_RED_THREADS / 32; i++) {
+      se += red[0][i];
+      sn += red[1][i];
+    }
     J.out[0] = se / sn;
     J.out[1] = sn;
   }
@@ -121,20 +216,21 @@ __global__ void energy_reduce_kernel(const EnJob *__restrict__ jobs, uint32_t n_
 
 void launch_energy_reduce(const EnJob *jobs, uint32_t n_jobs, const double *partials, void *stream) {
   if (n_jobs == 0) return;
-  const int warps = 4;
-  energy_reduce_kernel<<<(n_jobs + warps - 1) / warps, warps * 32, 0, (cudaStream_t)stream>>>(jobs, n_jobs,
-                                                                                           partials);
+  energy_reduce_kernel<<<n_jobs, EN_RED_THREADS, 0, (cudaStream_t)stream>>>(jobs, (const double2 *)partials);
 }
 
-void launch_energy(bool fp64, const EnJob *jobs, uint32_t n_jobs, uint32_t total_blocks,
-                   const EnClass *classes, const EnTerm *terms, double *partials, void *stream) {
+void launch_energy(bool fp64, bool pair, const EnTables &t, uint32_t n_jobs, uint32_t total_blocks, uint32_t rep_bits,
+                   void *stream) {
   if (n_jobs == 0 || total_blocks == 0) return;
   cudaStream_t s = (cudaStream_t)stream;
+  const unsigned threads = 1u << rep_bits;
   if (fp64)
-    energy_kernel<double><<<total_blocks, EN_THREADS, 0, s>>>(jobs, n_jobs, classes, terms, partials);
+    energy_kernel<double, false><<<total_blocks, threads, 0, s>>>(t, n_jobs);
+  else if (pair)
+    energy_kernel<float, true><<<total_blocks, threads, 0, s>>>(t, n_jobs);
   else
-    energy_kernel<float><<<total_blocks, EN_THREADS, 0, s>>>(jobs, n_jobs, classes, terms, partials);
-  launch_energy_reduce(jobs, n_jobs, partials, stream);
+    energy_kernel<float, false><<<total_blocks, threads, 0, s>>>(t, n_jobs);
+  launch_energy_reduce(t.jobs, n_jobs, t.partials, stream);
 }
 
 // ---------------------------------------------------------------------------

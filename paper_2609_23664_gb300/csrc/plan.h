@@ -136,9 +136,8 @@ struct FrameGroup {
 };
 
 struct HamLayout {
-  uint32_t n_eff = 0, chunk_bits = 0, n_blocks = 0;
-  std::vector<EnClass> classes;
-  std::vector<EnTerm> terms;
+  uint32_t n_eff = 0;
+  EnLayout en;
 };
 
 struct Engine;

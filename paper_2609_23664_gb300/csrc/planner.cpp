@@ -982,8 +982,10 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
     if (it != ham_ids.end()) { P->tasks[t].ham = it->second; continue; }
     HamLayout H;
     H.n_eff = n_eff;
-    build_energy_layout(T.terms.data(), T.terms.size(), n_eff, amp_bytes, &H.chunk_bits, H.classes, H.terms,
-                        &H.n_blocks);
+    // (energy blocks inside the persistent launch run in its 128-thread CTAs)
+    const bool fp64 = T.mode == QW_MODE_SV_FP64;
+    H.en = build_energy_layout(T.terms.data(), T.terms.size(), n_eff, fp64, !fp64,
+                               P->opts.fuse_energy ? 7u : en_rep_bits(n_eff));
     P->hams.push_back(std::move(H));
     ham_ids[key] = (int)P->hams.size() - 1;
     P->tasks[t].ham = ham_ids[key];

@@ -234,27 +234,66 @@ bool gate_matrix_1q(const qw_gate &g, double m[8], bool *diagonal);
 // ---------------------------------------------------------------------------
 // energy descriptors
 // ---------------------------------------------------------------------------
-struct EnTerm {
-  uint32_t xm, zm, skip, flags;  // flags bit0: imaginary component of conj(p)*a
-  double coef;                   // c_k * sign(i^{#Y}) * (2 if xm != 0)
+struct alignas(16) EnTerm {
+  uint32_t zm;
+  // bits 0-3: the term's mask as a combination of its group's basis; bit 4:
+  // imaginary component of conj(p)*a; bit 5 (pair layouts): it flips bit 0
+  // too; bits 8-11: parity of each basis vector under zm; EN_LAST_SIGN: the
+  // parity of the highest basis vector, for a term without flips
+  uint32_t code;
+  union {  // c_k * sign(i^{#Y}) * (2 if it flips), in the state's precision
+    double coef64;
+    float coef32;
+  };
+  // +-1 of the parities under zm of the directions (bit 0 of a pair layout,
+  // then the basis vectors) other than the pair's highest flipped one,
+  // ascending
+  float sign[4];
 };
-static_assert(sizeof(EnTerm) == 24, "EnTerm is read as two 8-byte words and a double");
-struct EnClass {
+constexpr uint32_t EN_LAST_SIGN = 1u << 12;
+static_assert(sizeof(EnTerm) == 32, "EnTerm is read as two 16-byte words");
+// Terms whose flip masks lie in the span of `basis` (independent vectors);
+// a coset is represented by its element with zeros at the four pivot bits
+// (a byte each in `pivots`, ascending).
+constexpr int EN_RANK = 4;
+constexpr uint32_t EN_GROUP_NORM = 1;   // flags: the group also sums the squared norm
+// flags above this bit: number of leading basis masks that have a term; the
+// group's first terms are one of each
+constexpr uint32_t EN_GROUP_SLOTS_SHIFT = 8;
+struct alignas(16) EnGroup {
+  uint32_t basis[EN_RANK];
+  uint32_t pivots;
   uint32_t term_begin, term_end;
-  uint32_t hb;           // highest bit of the class's flip pattern, 0xFFFFFFFF for class 0
-  uint32_t n_own;        // own chunks
+  uint32_t flags;
+};
+static_assert(sizeof(EnGroup) == 32, "EnGroup is read as two 16-byte words");
+// Groups of terms with the same flipped bits above the chunk size.
+struct EnClass {
+  uint32_t group_begin, group_end;
   uint32_t block_begin;  // first block of this class within its Hamiltonian layout
   uint32_t pad;
 };
 struct EnJob {
   const void *state;
   double *out;                     // {energy, norm2}
-  uint32_t n, chunk_bits;
+  uint32_t n;
+  uint32_t rep_bits, iter_bits;    // a block takes 2^rep_bits coset representatives 2^iter_bits times
   uint32_t class_begin, n_classes;
   uint32_t block_begin, n_blocks;  // global block range of this job
+  uint32_t pad;
 };
-constexpr int EN_THREADS = 256;
-constexpr int EN_BLOCK_BITS = 12;  // amplitudes per block: EN_THREADS x 16
+struct EnTables {
+  const EnJob *jobs;
+  const EnClass *classes;
+  const EnGroup *groups;
+  const EnTerm *terms;
+  double *partials;
+};
+// Representatives (threads) per block of the stand-alone launch: 128, fewer
+// on small registers so that one state still spreads over the SMs (a
+// 12-qubit state is 256 representatives in all)
+constexpr int EN_THREADS = 128;  // the largest block
+QW_HD constexpr uint32_t en_rep_bits(uint32_t n) { return n >= 18 ? 7 : (n >= 14 ? 6 : 5); }
 
 // ---------------------------------------------------------------------------
 // sampling descriptors
@@ -276,9 +315,24 @@ struct SmpShot {
 // the chunk size, so that one class touches pairs of chunks only.  Chunks
 // hold at most EN_CHUNK_BYTES of amplitudes of amp_bytes each.
 constexpr uint64_t EN_CHUNK_BYTES = 32ull << 20;
-void build_energy_layout(const qw_pauli_term *terms, uint64_t n_terms, uint32_t n, uint32_t amp_bytes,
-                         uint32_t *chunk_bits, std::vector<EnClass> &classes,
-                         std::vector<EnTerm> &en_terms, uint32_t *n_blocks);
+// Blocks go over several runs of representatives once a class has more than
+// 8192 of them: fewer partial sums to write and reduce (a 26-qubit state with
+// 16 classes left 262144 of them).  Runs further apart than that spread the
+// CTAs of a class over its chunks: 100 terms at 26 qubits 1.80 ms with 8192
+// blocks per class, 2.29 ms with 2048
+QW_HD constexpr uint32_t en_iter_bits(uint32_t n, uint32_t rep_bits) {
+  return n > EN_RANK + rep_bits + 13 ? n - EN_RANK - rep_bits - 13 : 0;
+}
+// FP32 states on a 16-byte boundary are read two amplitudes at a time
+inline bool en_pair(bool fp64, const void *state) { return !fp64 && ((uintptr_t)state & 15u) == 0; }
+struct EnLayout {
+  std::vector<EnClass> classes;
+  std::vector<EnGroup> groups;
+  std::vector<EnTerm> terms;
+  uint32_t rep_bits = 0, iter_bits = 0, n_blocks = 0;
+};
+EnLayout build_energy_layout(const qw_pauli_term *terms, uint64_t n_terms, uint32_t n, bool fp64, bool pair,
+                             uint32_t rep_bits, uint32_t max_class_bits = 32);
 
 // ---------------------------------------------------------------------------
 // tableau program (inverse-tableau formulation)
@@ -369,12 +423,6 @@ struct SvJob {
 struct SvSeg {
   uint32_t job, first;
 };
-struct EnTables {
-  const EnJob *jobs;
-  const EnClass *classes;
-  const EnTerm *terms;
-  double *partials;
-};
 
 // kernel attributes (dynamic shared memory limits); the first failure is returned
 cudaError_t sv_init_attrs();
@@ -390,16 +438,18 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
 // [2..] = per-job completed units (all zeroed by the caller beforehand).
 // Energy jobs need 128-thread CTAs (sv_threads_for_k(k_max) == 128).  ar:
 // SV_AR_PLAIN or SV_AR_COMP (FP32 states; SV_AR_REM is taken as PLAIN).
+// en.jobs: non-NULL when the list holds energy jobs.
 void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSeg *segs, uint32_t seg_bits,
                      uint32_t total_items, uint32_t k_max, unsigned int *counters, const EnTables &en,
                      int grid, void *stream, int ar = SV_AR_PLAIN);
-int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar = SV_AR_PLAIN);
+int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar = SV_AR_PLAIN, bool energy = false);
 void launch_copy(const void *src, void *dst, size_t bytes, void *stream);
 
 // energy: per-block partials (2 doubles per block), then one reduction
 // kernel writes {energy, norm2} of every job
-void launch_energy(bool fp64, const EnJob *jobs, uint32_t n_jobs, uint32_t total_blocks,
-                   const EnClass *classes, const EnTerm *terms, double *partials, void *stream);
+// (pair: the jobs' layouts and states, see en_pair)
+void launch_energy(bool fp64, bool pair, const EnTables &t, uint32_t n_jobs, uint32_t total_blocks, uint32_t rep_bits,
+                   void *stream);
 // the reduction alone, for partials written by the persistent launch
 void launch_energy_reduce(const EnJob *jobs, uint32_t n_jobs, const double *partials, void *stream);
 // sampling: block sums -> per-source sequential offsets -> shots

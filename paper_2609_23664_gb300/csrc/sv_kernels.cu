@@ -609,7 +609,9 @@ constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;  // 2 s per dependency wait
 // the 128-register build (MINB 4) can use.  Compensated passes (AR =
 // SV_AR_COMP) hold two FP32 complex values per amplitude in registers, 16
 // amplitudes per stage group, and are budgeted for three CTAs.
-template <typename T, int MINB, int AR, int NT>
+// EN: the work list may hold energy blocks (option fuse_energy); their code
+// stays out of the ordinary build, whose registers it would spill.
+template <typename T, int MINB, int AR, int NT, bool EN>
 __global__ void __launch_bounds__(NT, MINB)
 sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restrict__ segs,
                 uint32_t seg_bits, uint32_t total, unsigned int *ctr, EnTables en) {
@@ -657,13 +659,15 @@ sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restr
       continue;
     }
     const SvJob job = jobs[s_job];
-    if (job.kind == SVJ_ENERGY) {
-      if constexpr (NT == 128) {  // energy work items run in 128-thread CTAs only
+    bool tile = true;
+    if constexpr (EN) {
+      if (job.kind == SVJ_ENERGY) {
+        tile = false;
         const EnJob J = en.jobs[job.pass];
-        energy_block<T, 128, false>(J, s_unit, en.classes, en.terms,
-                                    en.partials + 2 * (size_t)(J.block_begin + s_unit));
+        energy_block<T, sizeof(T) == 4, false>(J, s_unit, en, en.partials + 2 * (size_t)(J.block_begin + s_unit));
       }
-    } else {
+    }
+    if (tile) {
       sv_tile<T, AR, sv_stage_width(AR, sizeof(T) == 8)>(t.passes + job.pass, t.stages, (const SvOpDesc<T> *)t.ops,
                                                          t.ops_lo, t.ph, (C *)smraw, (const C *)job.src,
                                                          (C *)job.dst, nullptr, nullptr, s_unit);
@@ -698,18 +702,17 @@ size_t sv_smem_bytes(bool fp64, uint32_t k, int ar) {
   return (size_t)(fp64 ? 16 : 8) << k << (ar == SV_AR_REM ? 1 : 0);
 }
 
-// the plain FP32 batch kernel for tiles of k qubits: with 32-amplitude
-// stages a 128-register build (four CTAs per SM) serves tiles of at most 12
-// qubits; 16-amplitude stages use one build
+// the batch kernel of a precision, arithmetic and tile width: plain FP32 has
+// a 128-register build (four CTAs per SM) for tiles of at most 12 qubits
 typedef void (*SvBatchKernel)(SvTables, const SvJob *, const SvSeg *, uint32_t, uint32_t, unsigned int *, EnTables);
-static SvBatchKernel plain32_batch(uint32_t k) {
-  if constexpr (SV_G_PLAIN32 == 4) {
-    (void)k;
-    return sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32>;
-  } else {
-    return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32>
-                  : sv_batch_kernel<float, 4, SV_AR_PLAIN, SV_NT_PLAIN32>;
-  }
+template <bool EN>
+static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar) {
+  if (fp64) return sv_batch_kernel<double, 1, SV_AR_PLAIN, 128, EN>;
+  if (ar == SV_AR_COMP) return sv_batch_kernel<float, 3, SV_AR_COMP, 128, EN>;
+  if constexpr (SV_G_PLAIN32 == 4) return sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, false>;
+  else
+    return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, EN>
+                  : sv_batch_kernel<float, 4, SV_AR_PLAIN, SV_NT_PLAIN32, EN>;
 }
 
 // Kernel attributes are set once, before any stream capture (a capture
@@ -720,10 +723,14 @@ cudaError_t sv_init_attrs() {
                      (const void *)sv_pass_kernel<float, SV_AR_COMP, 128, 3>,
                      (const void *)sv_pass_kernel<float, SV_AR_REM, 256, 1>,
                      (const void *)sv_pass_kernel<double, SV_AR_PLAIN, 128, 1>,
-                     (const void *)plain32_batch(13),
-                     (const void *)plain32_batch(12),
-                     (const void *)sv_batch_kernel<float, 3, SV_AR_COMP, 128>,
-                     (const void *)sv_batch_kernel<double, 1, SV_AR_PLAIN, 128>};
+                     (const void *)batch_kernel_of<false>(false, 13, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<false>(false, 12, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<false>(false, 13, SV_AR_COMP),
+                     (const void *)batch_kernel_of<false>(true, 13, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<true>(false, 13, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<true>(false, 12, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<true>(false, 13, SV_AR_COMP),
+                     (const void *)batch_kernel_of<true>(true, 13, SV_AR_PLAIN)};
   for (const void *f : k) {
     const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     if (e != cudaSuccess) return e;
@@ -755,18 +762,13 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
   }
 }
 
-int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar) {
+int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy) {
   if (fp64 || ar == SV_AR_REM) ar = SV_AR_PLAIN;
   const int threads = sv_threads_for_k(k, ar, fp64);
   const size_t smem = sv_smem_bytes(fp64, k, ar);
   int per_sm = 0;
-  if (fp64)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sv_batch_kernel<double, 1, SV_AR_PLAIN, 128>, threads,
-                                                  smem);
-  else if (ar == SV_AR_COMP)
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sv_batch_kernel<float, 3, SV_AR_COMP, 128>, threads, smem);
-  else
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, plain32_batch(k), threads, smem);
+  const SvBatchKernel f = energy ? batch_kernel_of<true>(fp64, k, ar) : batch_kernel_of<false>(fp64, k, ar);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem);
   if (per_sm < 1) per_sm = 1;
   return per_sm * sm_count;
 }
@@ -777,15 +779,9 @@ void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSe
   if (fp64 || ar == SV_AR_REM) ar = SV_AR_PLAIN;
   const int threads = sv_threads_for_k(k_max, ar, fp64);
   const size_t smem = sv_smem_bytes(fp64, k_max, ar);
-  cudaStream_t s = (cudaStream_t)stream;
-  if (fp64)
-    sv_batch_kernel<double, 1, SV_AR_PLAIN, 128><<<grid, threads, smem, s>>>(t, jobs, segs, seg_bits, total_items,
-                                                                             counters, en);
-  else if (ar == SV_AR_COMP)
-    sv_batch_kernel<float, 3, SV_AR_COMP, 128><<<grid, threads, smem, s>>>(t, jobs, segs, seg_bits, total_items,
-                                                                           counters, en);
-  else
-    plain32_batch(k_max)<<<grid, threads, smem, s>>>(t, jobs, segs, seg_bits, total_items, counters, en);
+  const SvBatchKernel f =
+      en.jobs ? batch_kernel_of<true>(fp64, k_max, ar) : batch_kernel_of<false>(fp64, k_max, ar);
+  f<<<grid, threads, smem, (cudaStream_t)stream>>>(t, jobs, segs, seg_bits, total_items, counters, en);
 }
 
 }  // namespace qw
