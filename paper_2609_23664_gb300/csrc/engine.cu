@@ -1635,6 +1635,21 @@ void engine_init(Engine *E, const qw_engine_opts *o) {
     cudaFree(a);
     cudaFree(b);
   }
+  // Workspaces of the calls on caller buffers come from a pool of the
+  // engine's own that keeps up to CALL_POOL_BYTES between calls (the device's
+  // default pool unmaps everything at each synchronization: a 24-qubit gate
+  // list then maps its 128 MB remainder array anew, 0.7 ms)
+  {
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = E->device;
+    cudaMemPool_t pool;
+    CK(cudaMemPoolCreate(&pool, &props));
+    E->call_pool = pool;
+    uint64_t keep = CALL_POOL_BYTES;
+    CK(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+  }
   // kernel attributes are set before any capture
   CK(sv_init_attrs());
   CK(tab_init_attrs());
@@ -1687,6 +1702,10 @@ void engine_release(Engine *E) {
   E->trim_cache();
   if (E->scratch) cudaFree(E->scratch);
   if (E->d_mlp) cudaFree(E->d_mlp);
+  if (E->call_pool) {
+    cudaDeviceSynchronize();  // its memory may still be in use on a caller's stream
+    cudaMemPoolDestroy((cudaMemPool_t)E->call_pool);
+  }
   if (E->stream) cudaStreamDestroy((cudaStream_t)E->stream);
 }
 
@@ -2066,13 +2085,34 @@ void costmodel_probe(Engine *E, const Workload &W, float *feat, float *tgt, floa
 // ---------------------------------------------------------------------------
 namespace qw {
 
-template <typename T>
-static T *stream_upload(const std::vector<T> &v, cudaStream_t s) {
-  T *p = nullptr;
-  CK(cudaMallocAsync((void **)&p, std::max<size_t>(16, v.size() * sizeof(T)), s));
-  if (!v.empty()) CK(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice, s));
-  return p;
-}
+// Host tables of one call, uploaded in one copy (each copy and allocation of
+// a small call costs more than its kernels).
+struct Blob {
+  std::vector<char> bytes;
+  template <typename T>
+  size_t add(const std::vector<T> &v) { return add(v.data(), v.size() * sizeof(T)); }
+  size_t add(const void *p, size_t n) {
+    const size_t at = (bytes.size() + 255) & ~(size_t)255;
+    bytes.resize(at + n);
+    if (n && p) memcpy(bytes.data() + at, p, n);
+    return at;
+  }
+};
+
+// Stream-ordered workspace of one call from the engine's pool: freed on the
+// same stream when the call's work is enqueued.
+struct CallSpace {
+  char *p = nullptr;
+  cudaStream_t s;
+  CallSpace(Engine *E, size_t bytes, cudaStream_t st) : s(st) {
+    CK(cudaMallocFromPoolAsync((void **)&p, std::max<size_t>(16, bytes), (cudaMemPool_t)E->call_pool, s));
+  }
+  CallSpace(const CallSpace &) = delete;
+  CallSpace &operator=(const CallSpace &) = delete;
+  ~CallSpace() {
+    if (p) cudaFreeAsync(p, s);
+  }
+};
 
 qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const qw_gate *gates,
                        uint64_t n_gates, bool init, void *stream) {
@@ -2097,30 +2137,25 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   SvTableBuilder tb(fp64);
   tb.add(pr);
   SvTables T;
-  SvPassDesc *dp = stream_upload(tb.passes, s);
-  SvStageDesc *ds = stream_upload(tb.stages, s);
-  void *dop = fp64 ? (void *)stream_upload(tb.ops64, s) : (void *)stream_upload(tb.ops32, s);
-  float *dlo = fp64 ? nullptr : stream_upload(tb.ops32lo, s);
-  float *dph = fp64 ? nullptr : stream_upload(tb.ph, s);
+  Blob bl;
+  const size_t op = bl.add(tb.passes), os = bl.add(tb.stages), oo = fp64 ? bl.add(tb.ops64) : bl.add(tb.ops32);
+  const size_t ol = bl.add(tb.ops32lo), oh = bl.add(tb.ph);
   const size_t np = pr.passes.size();
-  void *rem = nullptr;
-  if (ar == SV_AR_REM && np > 1) CK(cudaMallocAsync(&rem, sv_state_bytes(false, n), s));
-  T.passes = dp;
-  T.stages = ds;
-  T.ops = dop;
-  T.ops_lo = dlo;
-  T.ph = dph;
+  const size_t tab_bytes = (bl.bytes.size() + 255) & ~(size_t)255;
+  const bool keep_rem = ar == SV_AR_REM && np > 1;
+  CallSpace ws(E, tab_bytes + (keep_rem ? sv_state_bytes(false, n) : 0), s);
+  CK(cudaMemcpyAsync(ws.p, bl.bytes.data(), bl.bytes.size(), cudaMemcpyHostToDevice, s));
+  T.passes = (const SvPassDesc *)(ws.p + op);
+  T.stages = (const SvStageDesc *)(ws.p + os);
+  T.ops = ws.p + oo;
+  T.ops_lo = (const float *)(ws.p + ol);
+  T.ph = (const float *)(ws.p + oh);
+  void *rem = keep_rem ? ws.p + tab_bytes : nullptr;
   for (size_t p = 0; p < np; p++)
     launch_sv_pass(fp64, T, (uint32_t)p, (uint32_t)pr.passes[p].q.size(), n,
                    (p == 0 && init) ? nullptr : state, state, s, ar, p > 0 ? rem : nullptr,
                    p + 1 < np ? rem : nullptr);
   CK(cudaGetLastError());
-  CK(cudaFreeAsync(dp, s));
-  CK(cudaFreeAsync(ds, s));
-  if (dph) CK(cudaFreeAsync(dph, s));
-  CK(cudaFreeAsync(dop, s));
-  if (dlo) CK(cudaFreeAsync(dlo, s));
-  if (rem) CK(cudaFreeAsync(rem, s));
   return QW_OK;
 }
 
@@ -2131,12 +2166,11 @@ qw_status sv_energy_dev(Engine *E, uint32_t mode, uint32_t n, const void *state,
   const bool fp64 = mode == QW_MODE_SV_FP64;
   const bool pair = en_pair(fp64, state);
   const EnLayout H = build_energy_layout(terms, n_terms, n, fp64, pair, en_rep_bits(n));
-  EnClass *dc = stream_upload(H.classes, s);
-  EnGroup *dg = stream_upload(H.groups, s);
-  EnTerm *dt = stream_upload(H.terms, s);
-  double *dout = nullptr, *dpart = nullptr;
-  CK(cudaMallocAsync((void **)&dout, 2 * sizeof(double), s));
-  CK(cudaMallocAsync((void **)&dpart, 2 * sizeof(double) * H.n_blocks, s));
+  Blob bl;
+  const size_t oc = bl.add(H.classes), og = bl.add(H.groups), ot = bl.add(H.terms), oj = bl.add(nullptr, sizeof(EnJob));
+  const size_t tab_bytes = (bl.bytes.size() + 255) & ~(size_t)255;
+  CallSpace ws(E, tab_bytes + 2 * sizeof(double) * ((size_t)H.n_blocks + 1), s);
+  double *dout = (double *)(ws.p + tab_bytes), *dpart = dout + 2;
   EnJob j{};
   j.state = state;
   j.out = dout;
@@ -2147,16 +2181,13 @@ qw_status sv_energy_dev(Engine *E, uint32_t mode, uint32_t n, const void *state,
   j.n_classes = (uint32_t)H.classes.size();
   j.block_begin = 0;
   j.n_blocks = H.n_blocks;
-  EnJob *dj = stream_upload(std::vector<EnJob>{j}, s);
-  launch_energy(fp64, pair, EnTables{dj, dc, dg, dt, dpart}, 1, H.n_blocks, H.rep_bits, s);
+  memcpy(bl.bytes.data() + oj, &j, sizeof(j));
+  CK(cudaMemcpyAsync(ws.p, bl.bytes.data(), bl.bytes.size(), cudaMemcpyHostToDevice, s));
+  const EnTables tab{(const EnJob *)(ws.p + oj), (const EnClass *)(ws.p + oc), (const EnGroup *)(ws.p + og),
+                     (const EnTerm *)(ws.p + ot), dpart};
+  launch_energy(fp64, pair, tab, 1, H.n_blocks, H.rep_bits, s);
   double res[2];
   CK(cudaMemcpyAsync(res, dout, sizeof(res), cudaMemcpyDeviceToHost, s));
-  CK(cudaFreeAsync(dc, s));
-  CK(cudaFreeAsync(dg, s));
-  CK(cudaFreeAsync(dt, s));
-  CK(cudaFreeAsync(dout, s));
-  CK(cudaFreeAsync(dpart, s));
-  CK(cudaFreeAsync(dj, s));
   CK(cudaStreamSynchronize(s));
   *energy = res[0];
   if (norm2) *norm2 = res[1];
@@ -2174,23 +2205,29 @@ qw_status sv_sample_dev(Engine *E, uint32_t mode, uint32_t n, const void *state,
   so.n = n;
   so.n_blocks = (n >= (uint32_t)SMP_BLOCK_BITS) ? (1u << (n - SMP_BLOCK_BITS)) : 1u;
   so.block_begin = 0;
-  uint64_t *dres = nullptr;
-  CK(cudaMallocAsync((void **)&dres, shots * sizeof(uint64_t), s));
-  std::vector<SmpShot> sh(shots);
-  for (uint32_t k = 0; k < shots; k++) { sh[k].u = u[k]; sh[k].source = 0; sh[k].out = dres + k; }
-  SmpSource *dsrc = stream_upload(std::vector<SmpSource>{so}, s);
-  SmpShot *dsh = stream_upload(sh, s);
-  double *bsum = nullptr, *boff = nullptr;
-  int32_t *blast = nullptr;
-  int64_t *lastnz = nullptr;
-  CK(cudaMallocAsync((void **)&bsum, so.n_blocks * sizeof(double), s));
-  CK(cudaMallocAsync((void **)&boff, (so.n_blocks + 1) * sizeof(double), s));
-  CK(cudaMallocAsync((void **)&blast, so.n_blocks * sizeof(int32_t), s));
-  CK(cudaMallocAsync((void **)&lastnz, sizeof(int64_t), s));
-  launch_sampling(fp64, dsrc, 1, so.n_blocks, bsum, blast, boff, lastnz, dsh, shots, s);
-  CK(cudaMemcpyAsync(out, dres, shots * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
-  for (void *p : {(void *)dres, (void *)dsrc, (void *)dsh, (void *)bsum, (void *)boff, (void *)blast, (void *)lastnz})
-    CK(cudaFreeAsync(p, s));
+  // one workspace: results, the call's tables, block sums and offsets
+  const size_t res_bytes = ((size_t)shots * sizeof(uint64_t) + 255) & ~(size_t)255;
+  const size_t sh_bytes = (size_t)shots * sizeof(SmpShot);
+  const size_t nb = so.n_blocks;
+  const size_t o_src = res_bytes, o_sh = o_src + 256, o_sum = (o_sh + sh_bytes + 255) & ~(size_t)255;
+  const size_t o_off = o_sum + nb * sizeof(double), o_last = o_off + (nb + 1) * sizeof(double);
+  const size_t o_blast = o_last + sizeof(int64_t), total = o_blast + nb * sizeof(int32_t);
+  CallSpace ws(E, total, s);
+  std::vector<char> up(256 + sh_bytes);
+  memcpy(up.data(), &so, sizeof(so));
+  SmpShot *sh = (SmpShot *)(up.data() + 256);
+  for (uint32_t k = 0; k < shots; k++) {
+    SmpShot q{};
+    q.u = u[k];
+    q.out = (uint64_t *)ws.p + k;
+    sh[k] = q;
+  }
+  CK(cudaMemcpyAsync(ws.p + o_src, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+  launch_sampling(fp64, (const SmpSource *)(ws.p + o_src), 1, so.n_blocks, (double *)(ws.p + o_sum),
+                  (int32_t *)(ws.p + o_blast), (double *)(ws.p + o_off), (int64_t *)(ws.p + o_last),
+                  (const SmpShot *)(ws.p + o_sh), shots, s);
+  CK(cudaGetLastError());
+  CK(cudaMemcpyAsync(out, ws.p, (size_t)shots * sizeof(uint64_t), cudaMemcpyDeviceToHost, s));
   CK(cudaStreamSynchronize(s));
   return QW_OK;
 }

@@ -9,10 +9,9 @@
 //
 // Sampling: p_x = |psi_x|^2 summed in FP64 into a CDF that is never written
 // out: per 4096-amplitude block a lane sums 128 contiguous probabilities and
-// the 32 lane sums are chained in lane order; block offsets are chained in
-// block order; a shot finds its block by binary search and its index by
-// rescanning that block in the same order, so the CDF it searches is
-// exactly the one whose block totals were chained.
+// the 32 lane sums are chained in lane order; block offsets are an FP64 scan;
+// a shot finds its block by binary search and its index by rescanning that
+// block with the additions of the block sums.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -259,11 +258,17 @@ template <> struct SmpAcc<double> {
   double v = 0.0;
   __device__ __forceinline__ void add(double p) { v += p; }
   __device__ __forceinline__ double value() const { return v; }
+  typedef double raw;  // the running sum as it is kept in shared memory
+  __device__ __forceinline__ raw get() const { return v; }
+  static __device__ __forceinline__ double value_of(const raw &r) { return r; }
 };
 template <> struct SmpAcc<float> {
   DFAcc a;
   __device__ __forceinline__ void add(float p) { a.add(p); }
   __device__ __forceinline__ double value() const { return a.value(); }
+  typedef float2 raw;
+  __device__ __forceinline__ raw get() const { return make_float2(a.hi, a.lo); }
+  static __device__ __forceinline__ double value_of(const raw &r) { return (double)r.x + (double)r.y; }
 };
 __device__ __forceinline__ float prob32(const float2 &v) { return fmaf(v.x, v.x, v.y * v.y); }
 __device__ __forceinline__ double prob32(const double2 &v) { return fma(v.x, v.x, v.y * v.y); }
@@ -314,55 +319,107 @@ __device__ __forceinline__ double chain_scan(double s, int ln) {
   return S;
 }
 
+// One warp per block; the lane sums of the CTA's blocks are chained by one
+// thread per block, all of them at once (the 31 dependent FP64 adds of a
+// chain cost a warp the same for one block as for 32, and at 1/64 of the
+// FP32 rate they showed beside the loads).
+constexpr int SMP_WARPS = 8;
 template <typename T>
-__global__ void smp_blocksum_kernel(const SmpSource *__restrict__ srcs, uint32_t n_src,
-                                    uint32_t total, double *bsum, int32_t *blast) {
+__global__ void __launch_bounds__(SMP_WARPS * 32)
+smp_blocksum_kernel(const SmpSource *__restrict__ srcs, uint32_t n_src, uint32_t total, double *bsum, int32_t *blast) {
   typedef typename V2o<T>::t C;
-  const uint32_t gb = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  __shared__ double ls[SMP_WARPS][33];
+  __shared__ int32_t ll[SMP_WARPS];
+  const uint32_t w = threadIdx.x / 32, gb = blockIdx.x * SMP_WARPS + w;
   const int ln = threadIdx.x & 31;
-  if (gb >= total) return;
-  const SmpSource S = srcs[find_source(srcs, n_src, gb)];
-  const uint32_t blk = gb - S.block_begin;
-  const uint32_t dim = 1u << S.n;
-  double s;
-  int32_t last;
-  lane_sums<T>((const C *)S.state, dim, blk << SMP_BLOCK_BITS, ln, &s, &last);
-  const double incl = chain_scan(s, ln);
-  int32_t l = last;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) l = max(l, __shfl_xor_sync(0xffffffffu, l, o));
-  if (ln == 31) bsum[gb] = incl;
-  if (ln == 0) blast[gb] = l;
+  if (gb < total) {
+    const SmpSource S = srcs[find_source(srcs, n_src, gb)];
+    const uint32_t blk = gb - S.block_begin;
+    double s;
+    int32_t last;
+    lane_sums<T>((const C *)S.state, 1u << S.n, blk << SMP_BLOCK_BITS, ln, &s, &last);
+    ls[w][ln] = s;
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (ln == 0) ll[w] = last;
+  }
+  __syncthreads();
+  const uint32_t b = blockIdx.x * SMP_WARPS + threadIdx.x;
+  if (threadIdx.x < SMP_WARPS && b < total) {
+    double S = ls[threadIdx.x][0];
+    for (int l = 1; l < 32; l++) S = S + ls[threadIdx.x][l];
+    bsum[b] = S;
+    blast[b] = ll[threadIdx.x];
+  }
 }
 
-// one thread per source: boff[b] = sum of blocks before b (sequential); the
-// entry after the last block is the total
-__global__ void smp_offsets_kernel(const SmpSource *__restrict__ srcs, uint32_t n_src,
-                                   const double *bsum, const int32_t *blast, double *boff,
-                                   int64_t *lastnz) {
-  const uint32_t s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n_src) return;
+// one CTA per source: boff[b] = sum of the blocks before b, the entry after
+// the last block is the total.  Each thread adds a run of blocks in order,
+// the runs' sums are scanned across the CTA.  (One thread per source, block
+// by block, took 1.87 ms for the 16384 blocks of 26 qubits.)
+constexpr int SMP_OFF_THREADS = 256;
+__global__ void __launch_bounds__(SMP_OFF_THREADS)
+smp_offsets_kernel(const SmpSource *__restrict__ srcs, const double *__restrict__ bsum,
+                   const int32_t *__restrict__ blast, double *boff, int64_t *lastnz) {
+  const uint32_t s = blockIdx.x, t = threadIdx.x;
   const SmpSource S = srcs[s];
+  double *o = boff + S.block_begin + s;  // n_blocks + 1 entries per source
+  const uint32_t run = (S.n_blocks + SMP_OFF_THREADS - 1) / SMP_OFF_THREADS;
+  const uint32_t b0 = min(t * run, S.n_blocks), b1 = min(b0 + run, S.n_blocks);
   double acc = 0;
   int64_t last = -1;
-  double *o = boff + S.block_begin + s;  // n_blocks + 1 entries per source
-  for (uint32_t b = 0; b < S.n_blocks; b++) {
-    o[b] = acc;
+#pragma unroll 8
+  for (uint32_t b = b0; b < b1; b++) {
     acc = acc + bsum[S.block_begin + b];
     const int32_t l = blast[S.block_begin + b];
     if (l >= 0) last = ((int64_t)b << SMP_BLOCK_BITS) + l;
   }
-  o[S.n_blocks] = acc;
-  lastnz[s] = last;
+  // exclusive scan of the runs' sums: within a warp, then of the warps
+  __shared__ double wsum[SMP_OFF_THREADS / 32];
+  __shared__ int64_t wlast[SMP_OFF_THREADS / 32];
+  double incl = acc;
+#pragma unroll
+  for (int d = 1; d < 32; d *= 2) {
+    const double up = __shfl_up_sync(0xffffffffu, incl, d);
+    if ((t & 31) >= (uint32_t)d) incl = incl + up;
+  }
+  double excl = __shfl_up_sync(0xffffffffu, incl, 1);
+  if ((t & 31) == 0) excl = 0;
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, d));
+  if ((t & 31) == 31) wsum[t >> 5] = incl;
+  if ((t & 31) == 0) wlast[t >> 5] = last;
+  __syncthreads();
+  double before = 0;
+  for (uint32_t w = 0; w < (t >> 5); w++) before = before + wsum[w];
+  acc = before + excl;
+#pragma unroll 8
+  for (uint32_t b = b0; b < b1; b++) {
+    o[b] = acc;
+    acc = acc + bsum[S.block_begin + b];
+  }
+  if (t == SMP_OFF_THREADS - 1) {
+    o[S.n_blocks] = before + incl;
+    for (int w = 0; w < SMP_OFF_THREADS / 32; w++) last = max(last, wlast[w]);
+    lastnz[s] = last;
+  }
 }
 
+// One warp per shot: binary search for its block, then the block's lane sums,
+// then the running sums of the lane's 128 probabilities.  Those are FP32 pairs
+// (FP64 for FP64 states), formed by that lane alone and left in shared
+// memory; the 32 lanes then compare four of them each with the target in
+// FP64 (compared one by one by a single lane, 128 times three FP64 adds at
+// 1/64 of the FP32 rate took 145 of the 177 us of 4096 shots).
+constexpr int SMP_SHOT_WARPS = 4;
 template <typename T>
-__global__ void smp_shot_kernel(const SmpSource *__restrict__ srcs, const SmpShot *__restrict__ shots,
-                                uint32_t n_shots, const double *boff, const int64_t *lastnz) {
+__global__ void __launch_bounds__(SMP_SHOT_WARPS * 32)
+smp_shot_kernel(const SmpSource *__restrict__ srcs, const SmpShot *__restrict__ shots,
+                uint32_t n_shots, const double *boff, const int64_t *lastnz) {
   typedef typename V2o<T>::t C;
-  const uint32_t sh = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
+  __shared__ typename SmpAcc<T>::raw run[SMP_SHOT_WARPS][SMP_PER_LANE];
+  const uint32_t w = threadIdx.x / 32, sh = blockIdx.x * SMP_SHOT_WARPS + w;
   const int ln = threadIdx.x & 31;
-  if (sh >= n_shots) return;
+  if (sh >= n_shots) return;  // whole warps; no block-wide barrier below
   const SmpShot Q = shots[sh];
   const SmpSource S = srcs[Q.source];
   const double *o = boff + S.block_begin + Q.source;
@@ -389,27 +446,40 @@ __global__ void smp_shot_kernel(const SmpSource *__restrict__ srcs, const SmpSho
   const double excl = __shfl_up_sync(0xffffffffu, incl, 1);
   const double lane_start = (ln == 0) ? 0.0 : excl;
   const unsigned hit = __ballot_sync(0xffffffffu, ob + incl > target);
-  if (hit == 0) {  // rounding left the target at the block end: last nonzero
-    if (ln == 0) *Q.out = (uint64_t)lastnz[Q.source];
+  if (hit == 0) {
+    // the rounding of the block offsets left the target at the block's end:
+    // its last outcome of nonzero probability
+    last = __reduce_max_sync(0xffffffffu, last);
+    if (ln == 0)
+      *Q.out = last >= 0 ? ((uint64_t)blk << SMP_BLOCK_BITS) + (uint64_t)last : (uint64_t)lastnz[Q.source];
     return;
   }
   const int L = __ffs(hit) - 1;
+  const uint32_t b0 = (blk << SMP_BLOCK_BITS) + (uint32_t)L * SMP_PER_LANE;
+  const uint32_t cnt = min((uint32_t)SMP_PER_LANE, dim > b0 ? dim - b0 : 0u);
   if (ln == L) {
-    const uint32_t b0 = (blk << SMP_BLOCK_BITS) + (uint32_t)L * SMP_PER_LANE;
     SmpAcc<T> pre;
-    uint64_t ans = (uint64_t)b0 + SMP_PER_LANE - 1;
-    int64_t last_pos = -1;
-    for (int i = 0; i < SMP_PER_LANE; i++) {
-      const uint32_t x = b0 + i;
-      if (x >= dim) break;
-      const auto p = prob32(psi[x]);
-      pre.add(p);
-      if (p > 0) last_pos = x;
-      if (ob + (lane_start + pre.value()) > target) { ans = x; last_pos = -2; break; }
+    for (uint32_t i = 0; i < cnt; i++) {
+      pre.add(prob32(psi[b0 + i]));
+      run[w][i] = pre.get();
     }
-    if (last_pos >= 0) ans = (uint64_t)last_pos;
-    *Q.out = ans;
   }
+  const double from = __shfl_sync(0xffffffffu, lane_start, L);
+  const int32_t lane_last = __shfl_sync(0xffffffffu, last, L);
+  __syncwarp();
+  for (uint32_t c = 0; c < cnt; c += 32) {
+    const uint32_t i = c + (uint32_t)ln;
+    const bool over = i < cnt && ob + (from + SmpAcc<T>::value_of(run[w][i])) > target;
+    const unsigned m = __ballot_sync(0xffffffffu, over);
+    if (m) {
+      if (ln == 0) *Q.out = (uint64_t)b0 + c + (uint32_t)(__ffs(m) - 1);
+      return;
+    }
+  }
+  // no running sum exceeds the target: the lane's last nonzero outcome
+  if (ln == 0)
+    *Q.out = lane_last >= 0 ? ((uint64_t)blk << SMP_BLOCK_BITS) + (uint64_t)lane_last
+                            : (uint64_t)b0 + SMP_PER_LANE - 1;
 }
 
 void launch_sampling(bool fp64, const SmpSource *srcs, uint32_t n_src, uint32_t total_blocks,
@@ -417,19 +487,18 @@ void launch_sampling(bool fp64, const SmpSource *srcs, uint32_t n_src, uint32_t 
                      const SmpShot *shots, uint32_t n_shots, void *stream) {
   if (n_src == 0) return;
   cudaStream_t s = (cudaStream_t)stream;
-  const int wpb = 4;
-  const uint32_t g1 = (total_blocks + wpb - 1) / wpb;
+  const uint32_t g1 = (total_blocks + SMP_WARPS - 1) / SMP_WARPS;
   if (fp64)
-    smp_blocksum_kernel<double><<<g1, wpb * 32, 0, s>>>(srcs, n_src, total_blocks, bsum, blast);
+    smp_blocksum_kernel<double><<<g1, SMP_WARPS * 32, 0, s>>>(srcs, n_src, total_blocks, bsum, blast);
   else
-    smp_blocksum_kernel<float><<<g1, wpb * 32, 0, s>>>(srcs, n_src, total_blocks, bsum, blast);
-  smp_offsets_kernel<<<(n_src + 127) / 128, 128, 0, s>>>(srcs, n_src, bsum, blast, boff, lastnz);
+    smp_blocksum_kernel<float><<<g1, SMP_WARPS * 32, 0, s>>>(srcs, n_src, total_blocks, bsum, blast);
+  smp_offsets_kernel<<<n_src, SMP_OFF_THREADS, 0, s>>>(srcs, bsum, blast, boff, lastnz);
   if (n_shots == 0) return;
-  const uint32_t g3 = (n_shots + wpb - 1) / wpb;
+  const uint32_t g3 = (n_shots + SMP_SHOT_WARPS - 1) / SMP_SHOT_WARPS;
   if (fp64)
-    smp_shot_kernel<double><<<g3, wpb * 32, 0, s>>>(srcs, shots, n_shots, boff, lastnz);
+    smp_shot_kernel<double><<<g3, SMP_SHOT_WARPS * 32, 0, s>>>(srcs, shots, n_shots, boff, lastnz);
   else
-    smp_shot_kernel<float><<<g3, wpb * 32, 0, s>>>(srcs, shots, n_shots, boff, lastnz);
+    smp_shot_kernel<float><<<g3, SMP_SHOT_WARPS * 32, 0, s>>>(srcs, shots, n_shots, boff, lastnz);
 }
 
 }  // namespace qw

@@ -163,6 +163,8 @@ const char *kind_name(uint32_t k);
 void features_for(const TaskData &t, uint64_t b, uint64_t e, uint32_t n_sharing, const TileConfig &tc,
                   double occupancy, float out[QW_MLP_IN]);
 
+constexpr uint64_t CALL_POOL_BYTES = 1ull << 30;  // kept between calls
+
 struct Engine {
   int device = 0;
   int sm_count = 0;
@@ -176,7 +178,9 @@ struct Engine {
   std::map<uint64_t, double> dense_ms;    // measured dense-block pass times (autotuner cache)
   CostModel cm;
   float *d_mlp = nullptr;  // device copy of the MLP params
-  // scratch for the *_dev entry points
+  // stream-ordered memory of the calls on caller buffers (cudaMemPool_t)
+  void *call_pool = nullptr;
+  // scratch of the cost probe and prediction
   void *scratch = nullptr;
   size_t scratch_bytes = 0;
   // Device-memory cache: blocks a plan releases are kept (by size) for the
