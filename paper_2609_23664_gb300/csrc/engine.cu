@@ -401,6 +401,7 @@ struct DeviceState {
   // boundary's first pass waits for its parent's last); empty = per-pass launches
   struct MatBatch {
     bool fp64 = false;
+    int ar = SV_AR_PLAIN;
     uint32_t k_max = 5, seg_bits = 0, total_items = 0;
     int grid = 0;
     size_t n_jobs = 0, ctr_words = 0;
@@ -453,6 +454,9 @@ struct DeviceState {
     arena.release();
   }
 };
+
+// remainder arrays that the boundaries of a plan may hold together
+constexpr uint64_t MAT_REM_BYTES = 2ull << 30;
 
 static size_t sv_state_bytes(bool fp64, uint32_t n_eff) { return (size_t)(fp64 ? 16 : 8) << n_eff; }
 
@@ -728,6 +732,7 @@ static void prepare(qw_plan *P) {
   // sibling boundaries run side by side.  Otherwise: pass by pass.
   {
     bool ok = P->opts.batched != 0;
+    uint64_t mat_rem = 0;  // remainder arrays of every boundary
     size_t n_sv = 0;
     for (const qw_dense_prog *dp : D->mat_dense)
       if (dp) ok = false;  // a dense-block boundary is launched block by block
@@ -736,10 +741,13 @@ static void prepare(qw_plan *P) {
       n_sv++;
       if (M.sv.passes.empty()) ok = false;
       if (M.parent >= 0 && P->mats[M.parent].mode != M.mode) ok = false;
-      // compensated FP32 boundaries keep their remainder between passes,
-      // which the persistent launch does not carry: pass by pass
-      if (M.mode == QW_MODE_SV_FP32 && D->ar_chain == SV_AR_REM) ok = false;
+      // compensated FP32 boundaries keep their remainder between passes, an
+      // array each in a persistent launch
+      if (M.mode == QW_MODE_SV_FP32 && D->ar_chain == SV_AR_REM && M.sv.passes.size() > 1)
+        mat_rem += sv_state_bytes(false, M.n_eff);
     }
+    // beyond a small share of the budget: one array, pass by pass
+    if (mat_rem > std::min<uint64_t>(MAT_REM_BYTES, E->task_budget / 8)) ok = false;
     // a single boundary is a chain of dependent passes: separate launches
     // serve it as well, without CTAs waiting on the previous pass
     if (ok && n_sv > 1) {
@@ -756,6 +764,12 @@ static void prepare(qw_plan *P) {
       for (uint32_t prec : {(uint32_t)QW_MODE_SV_FP32, (uint32_t)QW_MODE_SV_FP64}) {
         std::vector<SvJob> jobs;
         std::vector<int> last_job(P->mats.size(), -1);
+        const int ar = prec == QW_MODE_SV_FP32 ? D->ar_chain : SV_AR_PLAIN;
+        std::vector<void *> rems(P->mats.size(), nullptr);
+        if (ar == SV_AR_REM)
+          for (size_t m = 0; m < P->mats.size(); m++)
+            if (P->mats[m].mode == prec && P->mats[m].sv.passes.size() > 1)
+              rems[m] = D->arena.alloc(sv_state_bytes(false, P->mats[m].n_eff));
         uint32_t kmax = 5;
         for (uint32_t L = 0; L <= max_level; L++)
           for (size_t pi = 0; pi < max_p; pi++)
@@ -771,6 +785,8 @@ static void prepare(qw_plan *P) {
               j.dep = (pi == 0) ? (M.parent >= 0 ? last_job[M.parent] : -1) : last_job[m];
               j.kind = SVJ_PASS;
               j.n = M.n_eff;
+              j.src_lo = pi > 0 ? rems[m] : nullptr;
+              j.dst_lo = pi + 1 < M.sv.passes.size() ? rems[m] : nullptr;
               last_job[m] = (int)jobs.size();
               jobs.push_back(j);
               kmax = std::max(kmax, k);
@@ -779,7 +795,8 @@ static void prepare(qw_plan *P) {
         DeviceState::MatBatch B;
         B.fp64 = prec == QW_MODE_SV_FP64;
         B.k_max = kmax;
-        B.grid = sv_batch_grid(B.fp64, kmax, E->sm_count);
+        B.ar = ar;
+        B.grid = sv_batch_grid(B.fp64, kmax, E->sm_count, ar);
         B.seg_bits = segment_bits(jobs);
         std::vector<SvSeg> segs;
         build_segments(jobs, jobs.size(), B.seg_bits, 2ull * (uint64_t)B.grid, segs);
@@ -835,49 +852,69 @@ static void prepare(qw_plan *P) {
   }
   size_t max_partials = 1, max_smp_blocks = 1, max_src = 1;
   const bool batched = P->opts.batched != 0;
-  // compensated FP32 tasks with long programs leave the persistent launch
-  // (which rounds at every stage) for a chain of launches of their own that
-  // keeps the remainder, one task after another
-  auto long_chain = [&](const TaskPlan &tp) {
-    return batched && D->ar_batch == SV_AR_COMP && tp.mode == QW_MODE_SV_FP32 &&
-           tp.sv.passes.size() > (size_t)SV_COMP_MAX_BATCH_PASSES;
+  // Compensated FP32 tasks with long programs keep their remainder between
+  // passes.  Where the tiles of one pass take at most half of the resident
+  // CTAs (up to 19 qubits), several tasks advance together in a persistent
+  // launch, each with its remainder array; larger registers fill the chip
+  // alone and run one after another, pass by pass.
+  auto long_chain = [&](const TaskPlan &tp) { return batched && tp.chain; };
+  const uint32_t rem_slots = (uint32_t)sv_batch_grid(false, SV_MAX_TILE_FP32_REM, E->sm_count, SV_AR_REM);
+  auto shares_launch = [&](const TaskPlan &tp) {
+    return !tp.sv.passes.empty() && 2u << (tp.n_eff - (uint32_t)tp.sv.passes[0].q.size()) <= rem_slots;
   };
   // Task buffers of every group coexist for the plan's lifetime, so the
   // groups share one task budget: each group with pooled tasks gets one
   // buffer, then the rest of the budget goes to the groups in order of
-  // state size (smallest first) for up to one buffer per pooled task.
-  std::map<std::pair<int, uint32_t>, size_t> pool_size;
+  // state size (smallest first) for up to one buffer per pooled task, and
+  // for up to one state and remainder per long chain.
+  std::map<std::pair<int, uint32_t>, size_t> pool_size, long_size;
   {
+    std::map<std::pair<int, uint32_t>, size_t> n_long;
+    std::map<std::pair<int, uint32_t>, bool> n_share;
     std::vector<std::pair<size_t, std::pair<int, uint32_t>>> order;  // (S, group)
     std::map<std::pair<int, uint32_t>, size_t> n_pooled;
     uint64_t committed = 0;
     for (auto &g : groups) {
-      size_t np = 0;
-      bool any_long = false;
+      size_t np = 0, nl = 0;
+      bool pooled_long = false;
       for (uint32_t t : g.second) {
         const TaskPlan &tp = P->tasks[t];
-        if ((!tp.sv.passes.empty() || needs_convert(tp)) && !(tp.flags & QW_TASK_KEEP_STATE)) {
-          if (long_chain(tp)) any_long = true;
-          else np++;
+        if (tp.sv.passes.empty() && !needs_convert(tp)) continue;
+        if (long_chain(tp)) {
+          nl++;
+          n_share[g.first] = shares_launch(tp);
+          pooled_long = pooled_long || !(tp.flags & QW_TASK_KEEP_STATE);
+        } else if (!(tp.flags & QW_TASK_KEEP_STATE)) {
+          np++;
         }
       }
-      if (any_long && np == 0) np = 1;
+      if (pooled_long && np == 0) np = 1;
       const size_t S = sv_state_bytes(g.first.first != 0, g.first.second);
       n_pooled[g.first] = np;
+      n_long[g.first] = nl;
       pool_size[g.first] = np ? 1 : 0;
-      if (np) {
-        committed += S;
-        order.push_back({S, g.first});
-      }
+      long_size[g.first] = nl ? 1 : 0;
+      if (np) committed += S;
+      if (nl) committed += S;  // the remainder of one chain
+      if (np || nl) order.push_back({S, g.first});
     }
     std::sort(order.begin(), order.end());
     uint64_t left = E->task_budget > committed ? E->task_budget - committed : 0;
     for (auto &o : order) {
       if (!batched) break;
       const size_t S = o.first;
-      const size_t extra = std::min<size_t>(n_pooled[o.second] - 1, (size_t)(left / S));
+      const size_t np = n_pooled[o.second], nl = n_long[o.second];
+      const size_t extra = std::min<size_t>(np ? np - 1 : 0, (size_t)(left / S));
       pool_size[o.second] += extra;
       left -= (uint64_t)extra * S;
+      // chains share the pooled states (their waves run at other times)
+      for (size_t k = 1; k < nl && n_share[o.second]; k++) {
+        const size_t need = S + (long_size[o.second] >= pool_size[o.second] ? S : 0);
+        if (left < need) break;
+        left -= need;
+        long_size[o.second]++;
+        pool_size[o.second] = std::max(pool_size[o.second], long_size[o.second]);
+      }
     }
   }
   for (auto &g : groups) {
@@ -907,10 +944,14 @@ static void prepare(qw_plan *P) {
       if (long_chain(P->tasks[t])) { longs.push_back(t); pooled_long = true; }
       else pool_short.push_back(t);
     }
-    const size_t pool_n =
-        std::min(pool_size[g.first], std::max(pool_short.size(), (size_t)(pooled_long ? 1 : 0)));
+    const size_t long_n = std::min(long_size[g.first], longs.size());
+    const size_t pool_n = std::min(pool_size[g.first], std::max(pool_short.size(), pooled_long ? long_n : (size_t)0));
     std::vector<void *> pool(pool_n);
     for (auto &p : pool) p = D->arena.alloc(S);
+    // remainder arrays of the chains of one wave (a single chain at a time
+    // shares the boundaries' array, as it is launched pass by pass)
+    std::vector<void *> rems(long_n > 1 ? long_n : 0);
+    for (auto &p : rems) p = D->arena.alloc(S);
     std::vector<std::pair<std::vector<uint32_t>, bool>> wave_tasks;  // (tasks, per-pass launches)
     if (batched) {
       if (!ded_short.empty()) wave_tasks.push_back({ded_short, false});
@@ -918,7 +959,10 @@ static void prepare(qw_plan *P) {
         wave_tasks.push_back({std::vector<uint32_t>(pool_short.begin() + i,
                                                     pool_short.begin() + std::min(pool_short.size(), i + pool_n)),
                               false});
-      for (uint32_t t : longs) wave_tasks.push_back({{t}, true});
+      const size_t lw = std::max<size_t>(1, long_n);
+      for (size_t i = 0; i < longs.size(); i += lw)
+        wave_tasks.push_back({std::vector<uint32_t>(longs.begin() + i, longs.begin() + std::min(longs.size(), i + lw)),
+                              lw == 1});
     } else {
       for (uint32_t t : own) wave_tasks.push_back({{t}, true});
     }
@@ -927,8 +971,9 @@ static void prepare(qw_plan *P) {
       Wave W;
       W.fp64 = fp64;
       W.per_pass = wave_tasks[w].second;
-      W.ar = fp64 ? SV_AR_PLAIN : (W.per_pass ? D->ar_chain : D->ar_batch);
       W.tasks = wave_tasks[w].first;
+      const bool chains = !W.tasks.empty() && long_chain(P->tasks[W.tasks[0]]);  // (a wave holds one kind)
+      W.ar = fp64 ? SV_AR_PLAIN : (W.per_pass || chains ? D->ar_chain : D->ar_batch);
       uint32_t kmax = 5;
       for (size_t i = 0; i < W.tasks.size(); i++) {
         const uint32_t t = W.tasks[i];
@@ -968,6 +1013,10 @@ static void prepare(qw_plan *P) {
             j.dep = last[i];
             j.kind = SVJ_PASS;
             j.n = tp.n_eff;
+            if (chains && !W.per_pass) {
+              j.src_lo = p > 0 ? rems[i] : nullptr;
+              j.dst_lo = p + 1 < tp.sv.passes.size() ? rems[i] : nullptr;
+            }
             last[i] = (int)W.jobs.size();
             last_pass[t] = (int)W.jobs.size();
             W.jobs.push_back(j);
@@ -1031,9 +1080,9 @@ static void prepare(qw_plan *P) {
       max_src = std::max<size_t>(max_src, W.src.size());
       // algorithmic bytes: every pass reads and writes its state once; the
       // energy of a task reads every amplitude once per term class
-      if (W.ar == SV_AR_REM) {  // one task, its passes in order
-        P->batch_alg_bytes += chain_bytes((double)S, W.jobs.size(), W.ar);
-        if (W.jobs.size() > 1) rem_bytes = std::max(rem_bytes, S);
+      if (W.ar == SV_AR_REM) {
+        for (uint32_t t : W.tasks) P->batch_alg_bytes += chain_bytes((double)S, P->tasks[t].sv.passes.size(), W.ar);
+        if (W.per_pass && W.jobs.size() > 1) rem_bytes = std::max(rem_bytes, S);
       } else {
         for (const SvJob &j : W.jobs) { (void)j; P->batch_alg_bytes += 2.0 * (double)S; }
       }
@@ -1048,7 +1097,7 @@ static void prepare(qw_plan *P) {
       // released in the order their states finish
       std::vector<SvJob> up = W.jobs;
       W.fused_energy =
-          !W.per_pass && P->opts.fuse_energy && !W.en.empty() && sv_threads_for_k(W.k_max, W.ar, fp64) == 128;
+          !W.per_pass && W.ar != SV_AR_REM && P->opts.fuse_energy && !W.en.empty() && sv_threads_for_k(W.k_max, W.ar, fp64) == 128;
       W.grid = !W.per_pass ? sv_batch_grid(fp64, W.k_max, E->sm_count, W.ar, W.fused_energy) : 0;
       if (W.fused_energy) {
         std::vector<SvJob> ej;
@@ -1334,7 +1383,7 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
     for (const DeviceState::MatBatch &B : D->mat_batches) {
       CK(cudaMemsetAsync(B.d_ctr, 0, B.ctr_words * sizeof(unsigned int), s));
       launch_sv_batch(B.fp64, B.fp64 ? D->t64 : D->t32, B.d_jobs, B.d_segs, B.seg_bits, B.total_items, B.k_max,
-                      B.d_ctr, EnTables{}, B.grid, s);
+                      B.d_ctr, EnTables{}, B.grid, s, B.ar);
       nl += 1;
     }
     // each boundary rounded once into the other precision its consumers use
@@ -1771,13 +1820,17 @@ TileConfig Engine::tile_config(uint32_t n_eff, bool fp64, int ar, uint32_t mix) 
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
-  const uint32_t ks32[3] = {12, 13, 14}, ks64[3] = {11, 12, 13}, bs[3] = {3, 4, 5};
+  const uint32_t ks32[5] = {12, 13, 14, 0, 0}, ks64[5] = {11, 12, 13, 9, 10}, bs[3] = {3, 4, 5};
   float best_ms = 1e30f;
   const uint32_t best_cap = best.k_max;
   // a register that fits one tile is timed with that single shape (its
   // per-pass time calibrates the analytic cost model)
-  const bool one_tile = key_n <= best.k_max;
-  for (int ki = 0; ki < 3; ki++) {
+  // Small FP64 registers are timed with smaller tiles too: a state that fits
+  // one tile runs on one SM, whose FP64 pipe (1/64 of the FP32 rate) it then
+  // waits for, 0.9 ms for a 6-layer 12-qubit prefix.
+  const bool small64 = fp64 && key_n <= 16;
+  const bool one_tile = key_n <= best.k_max && !(small64 && key_n >= 11);
+  for (int ki = 0; ki < (small64 ? 5 : 3); ki++) {
     for (int bi = 0; bi < 3; bi++) {
       TileConfig tc;
       tc.k_max = fp64 ? ks64[ki] : ks32[ki];
@@ -2125,6 +2178,7 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   uint64_t n2 = 0;
   for (uint64_t i = 0; i < n_gates; i++) n2 += is_two_qubit_op(gates[i].op) ? 1 : 0;
   TileConfig tc = E->tile_config(n, fp64, SV_AR_COMP, gate_mix(n2, n_gates));
+  tc.k_max = std::min<uint32_t>(tc.k_max, sv_max_tile(ar, fp64));
   SvProgram pr = fuse_sv(gates, n_gates, n, tc);
   if (pr.passes.empty()) {
     if (!init) return QW_OK;

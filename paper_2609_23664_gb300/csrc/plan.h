@@ -116,6 +116,7 @@ struct TaskPlan {
   int ham = -1;             // Hamiltonian layout id, -1 = no energy
   std::vector<double> uniforms;
   SvProgram sv;             // suffix program (SV modes)
+  bool chain = false;       // compensated FP32 passes that keep their remainder (SV_AR_REM)
   std::vector<std::pair<uint32_t, uint32_t>> tab_segs;
   uint32_t tab_outs = 0;    // suffix outcomes
   uint32_t total_outs = 0;  // all MEASURE outcomes of the task

@@ -443,14 +443,15 @@ struct PlanCtx {
     return mix_of[key] = gate_mix(n2, all);
   }
 
-  TileConfig tiles(uint32_t n_eff, bool fp64) {
+  // chain: for passes that keep their remainder (compensated FP32)
+  TileConfig tiles(uint32_t n_eff, bool fp64, bool chain = false) {
     TileConfig tc;
     tc.k_max = fp64 ? 12 : 13;
     tc.b = 4;
     const int ar = fp64 ? SV_AR_PLAIN : plan_ar_batch(P);
     tc.g = sv_stage_width(ar, fp64);
     if (E) tc = E->tile_config(n_eff, fp64, ar, mix(n_eff, fp64));
-    const uint32_t kcap = sv_max_tile(ar, fp64);
+    const uint32_t kcap = sv_max_tile(chain && ar == SV_AR_COMP ? SV_AR_REM : ar, fp64);
     if (P->opts.tile_qubits) tc.k_max = std::min<uint32_t>(P->opts.tile_qubits, kcap);
     tc.k_max = std::min<uint32_t>(tc.k_max, kcap);
     if (P->opts.low_qubits) tc.b = P->opts.low_qubits;
@@ -1030,7 +1031,7 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
       M.out_offset = (M.parent >= 0) ? P->mats[M.parent].out_offset + P->mats[M.parent].tab_outs : 0;
     } else {
       R.copy_gates(M.begin, M.end, buf);
-      TileConfig tc = C.tiles(M.n_eff, M.mode == QW_MODE_SV_FP64);
+      TileConfig tc = C.tiles(M.n_eff, M.mode == QW_MODE_SV_FP64, true);
       M.sv = fuse_sv(buf.data(), buf.size(), M.n_eff, tc);
       if (P->opts.dense_boundaries) M.gates = buf;
     }
@@ -1046,6 +1047,12 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
       T.copy_gates(tp.begin, T.n_gates, buf);
       TileConfig tc = C.tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
       tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc);
+      tp.chain = T.mode == QW_MODE_SV_FP32 && plan_ar_batch(P) == SV_AR_COMP &&
+                 (!P->opts.batched || tp.sv.passes.size() > (size_t)SV_COMP_MAX_BATCH_PASSES);
+      if (tp.chain) {
+        tc = C.tiles(tp.n_eff, false, true);
+        tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc);
+      }
       if (tp.sv.passes.empty() && tp.src < 0) {
         // no gates at all: one pass without stages materializes |0...0>
         HostPass hp;

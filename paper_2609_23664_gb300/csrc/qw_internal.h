@@ -100,12 +100,17 @@ __host__ __device__ constexpr uint32_t sv_op_index(uint32_t kind, uint32_t a, ui
 }
 constexpr int SV_MAX_TILE_FP32 = 14;
 constexpr int SV_MAX_TILE_FP64 = 13;
-// compensated FP32 passes keep a remainder plane beside the tile (16 bytes
-// of shared memory per amplitude), so their tiles stop at 2^13
+// compensated FP32 passes run four-position stages, whose descriptor holds
+// the group bits of tiles up to 2^13
 constexpr int SV_MAX_TILE_FP32_COMP = 13;
-// a compensated FP32 task whose program has more passes than this runs as
-// its own chain of launches that keeps the remainder (persistent launches
-// round at every stage, which suits short suffixes only)
+// chains that keep their remainder between passes hold it in a plane beside
+// the tile (16 bytes of shared memory per amplitude): 2^12 amplitudes leave
+// three CTAs per SM, 2^13 one (200 random gates at 24 qubits: 2.83 against
+// 3.58 ms)
+constexpr int SV_MAX_TILE_FP32_REM = 12;
+// a compensated FP32 task whose program has more passes than this keeps its
+// remainder between passes (rounding at every stage suits short suffixes
+// only)
 constexpr uint32_t SV_COMP_MAX_BATCH_PASSES = 8;
 
 struct HostOp {
@@ -402,7 +407,9 @@ QW_HD constexpr int sv_stage_width(int ar, bool fp64 = false) {
 }
 // largest tile of those passes (a stage's group bits are at most SV_MAX_GBITS)
 QW_HD constexpr int sv_max_tile(int ar, bool fp64) {
-  return fp64 ? SV_MAX_TILE_FP64 : (sv_stage_width(ar, fp64) == 4 ? SV_MAX_TILE_FP32_COMP : SV_MAX_TILE_FP32);
+  return fp64 ? SV_MAX_TILE_FP64
+         : ar == SV_AR_REM ? SV_MAX_TILE_FP32_REM
+                           : (sv_stage_width(ar, fp64) == 4 ? SV_MAX_TILE_FP32_COMP : SV_MAX_TILE_FP32);
 }
 // A job of the persistent launch: one pass over one state (n_tiles tiles),
 // or the energy blocks of one state (kind SVJ_ENERGY, n_tiles blocks).
@@ -410,6 +417,9 @@ enum SvJobKind : uint32_t { SVJ_PASS = 0, SVJ_ENERGY = 1 };
 struct SvJob {
   const void *src;   // NULL: start from |0...0>
   void *dst;
+  // SV_AR_REM launches: remainder arrays read and written (NULL: zero, dropped)
+  const void *src_lo;
+  void *dst_lo;
   uint32_t pass;     // SVJ_PASS: index into the pass table; SVJ_ENERGY: index of the EnJob
   uint32_t n_tiles;  // work units
   int32_t dep;       // job that must finish first, -1 none
@@ -437,7 +447,7 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
 // persistent batch over jobs; counters: [0] = next item, [1] = error flag,
 // [2..] = per-job completed units (all zeroed by the caller beforehand).
 // Energy jobs need 128-thread CTAs (sv_threads_for_k(k_max) == 128).  ar:
-// SV_AR_PLAIN or SV_AR_COMP (FP32 states; SV_AR_REM is taken as PLAIN).
+// of FP32 states (energy jobs: not with SV_AR_REM).
 // en.jobs: non-NULL when the list holds energy jobs.
 void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSeg *segs, uint32_t seg_bits,
                      uint32_t total_items, uint32_t k_max, unsigned int *counters, const EnTables &en,

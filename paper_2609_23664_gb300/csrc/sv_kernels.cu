@@ -670,7 +670,8 @@ sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restr
     if (tile) {
       sv_tile<T, AR, sv_stage_width(AR, sizeof(T) == 8)>(t.passes + job.pass, t.stages, (const SvOpDesc<T> *)t.ops,
                                                          t.ops_lo, t.ph, (C *)smraw, (const C *)job.src,
-                                                         (C *)job.dst, nullptr, nullptr, s_unit);
+                                                         (C *)job.dst, (const float2 *)job.src_lo,
+                                                         (float2 *)job.dst_lo, s_unit);
     }
     // every thread's writes of the unit precede thread 0's release through
     // the barrier (bar.sync orders them at CTA scope; the fence is
@@ -689,13 +690,12 @@ sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restr
 // (FP32) or five (FP64) positions.  Threads: every thread owns at least two
 // stage groups of a 2^13 tile (128 threads; 256 for plain FP32 passes with
 // four-position stages, whose register budget fits three such CTAs per
-// SM); passes with a remainder plane (twice the shared memory, one CTA per
-// SM) give every stage group its own thread, up to 256.
+// SM).
 constexpr int SV_NT_PLAIN32 = (SV_G_PLAIN32 == 4) ? 256 : 128;
 int sv_threads_for_k(uint32_t k, int ar, bool fp64) {
   const uint32_t G = (uint32_t)sv_stage_width(ar, fp64);
-  const uint32_t g = (ar == SV_AR_REM) ? 1u << (k - G) : 1u << (k - G - 1);
-  const uint32_t cap = (ar == SV_AR_REM) ? 256u : (!fp64 && ar == SV_AR_PLAIN) ? (uint32_t)SV_NT_PLAIN32 : 128u;
+  const uint32_t g = 1u << (k - G - 1);
+  const uint32_t cap = (!fp64 && ar == SV_AR_PLAIN) ? (uint32_t)SV_NT_PLAIN32 : 128u;
   return (int)(g < 32 ? 32 : (g > cap ? cap : g));
 }
 size_t sv_smem_bytes(bool fp64, uint32_t k, int ar) {
@@ -709,6 +709,7 @@ template <bool EN>
 static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar) {
   if (fp64) return sv_batch_kernel<double, 1, SV_AR_PLAIN, 128, EN>;
   if (ar == SV_AR_COMP) return sv_batch_kernel<float, 3, SV_AR_COMP, 128, EN>;
+  if (ar == SV_AR_REM) return sv_batch_kernel<float, 3, SV_AR_REM, 128, false>;
   if constexpr (SV_G_PLAIN32 == 4) return sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, false>;
   else
     return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, EN>
@@ -721,12 +722,13 @@ cudaError_t sv_init_attrs() {
   const int bytes = 200 * 1024;
   const void *k[] = {(const void *)sv_pass_kernel<float, SV_AR_PLAIN, SV_NT_PLAIN32, 3>,
                      (const void *)sv_pass_kernel<float, SV_AR_COMP, 128, 3>,
-                     (const void *)sv_pass_kernel<float, SV_AR_REM, 256, 1>,
+                     (const void *)sv_pass_kernel<float, SV_AR_REM, 128, 3>,
                      (const void *)sv_pass_kernel<double, SV_AR_PLAIN, 128, 1>,
                      (const void *)batch_kernel_of<false>(false, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 12, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 13, SV_AR_COMP),
                      (const void *)batch_kernel_of<false>(true, 13, SV_AR_PLAIN),
+                     (const void *)batch_kernel_of<false>(false, 12, SV_AR_REM),
                      (const void *)batch_kernel_of<true>(false, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<true>(false, 12, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<true>(false, 13, SV_AR_COMP),
@@ -751,7 +753,7 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
     sv_pass_kernel<double, SV_AR_PLAIN, 128, 1><<<tiles, threads, smem, s>>>(t, pass_idx, (const double2 *)src,
                                                                               (double2 *)dst, nullptr, nullptr);
   } else if (ar == SV_AR_REM) {
-    sv_pass_kernel<float, SV_AR_REM, 256, 1><<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src,
+    sv_pass_kernel<float, SV_AR_REM, 128, 3><<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src,
                                                                            (float2 *)dst, sl, dl);
   } else if (ar == SV_AR_COMP) {
     sv_pass_kernel<float, SV_AR_COMP, 128, 3><<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src,
@@ -763,7 +765,7 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
 }
 
 int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy) {
-  if (fp64 || ar == SV_AR_REM) ar = SV_AR_PLAIN;
+  if (fp64) ar = SV_AR_PLAIN;
   const int threads = sv_threads_for_k(k, ar, fp64);
   const size_t smem = sv_smem_bytes(fp64, k, ar);
   int per_sm = 0;
@@ -776,7 +778,7 @@ int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy) {
 void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSeg *segs, uint32_t seg_bits,
                      uint32_t total_items, uint32_t k_max, unsigned int *counters, const EnTables &en,
                      int grid, void *stream, int ar) {
-  if (fp64 || ar == SV_AR_REM) ar = SV_AR_PLAIN;
+  if (fp64) ar = SV_AR_PLAIN;
   const int threads = sv_threads_for_k(k_max, ar, fp64);
   const size_t smem = sv_smem_bytes(fp64, k_max, ar);
   const SvBatchKernel f =
