@@ -10,7 +10,7 @@
 // Sums run in FP32 in ascending index order.  The backward pass treats the
 // roundings as identities (straight-through) and returns gradients of
 // mean (y - t)^2 with respect to the FP32 master parameters.  Per-CTA
-// gradient partials are reduced in CTA order, so results are deterministic.
+// gradient partials are reduced in a fixed order, so results are deterministic.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -22,7 +22,16 @@ constexpr int MI = QW_MLP_IN, MH = QW_MLP_HID;
 constexpr int OFF_W1 = 0, OFF_B1 = MI * MH, OFF_W2 = OFF_B1 + MH, OFF_B2 = OFF_W2 + MH * MH,
               OFF_W3 = OFF_B2 + MH, OFF_B3 = OFF_W3 + MH, N_PARAMS = OFF_B3 + 1;
 static_assert(N_PARAMS == QW_MLP_PARAMS, "parameter layout");
-constexpr int MLP_SPB = 32;  // samples per CTA
+// Samples run one after another in a CTA of 64 threads, so a batch is spread
+// over up to 100 CTAs (a 256-sample gradient took 55 us on 8 CTAs of 32
+// samples); their gradient partials, 20 KB each, then still fit the 2 MB that
+// the allocator maps at a time.
+constexpr uint32_t MLP_MAX_CTAS = 100;
+static uint32_t mlp_spb(uint32_t batch) { return (batch + MLP_MAX_CTAS - 1) / MLP_MAX_CTAS; }
+static uint32_t mlp_ctas(uint32_t batch) {
+  const uint32_t spb = mlp_spb(batch);
+  return spb ? (batch + spb - 1) / spb : 0;
+}
 
 __device__ __forceinline__ float bf(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
@@ -30,8 +39,9 @@ __device__ __forceinline__ float bf(float v) { return __bfloat162float(__float2b
 template <bool BACKWARD>
 __global__ void __launch_bounds__(MH)
 mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float *__restrict__ Tg,
-           float *__restrict__ Y, uint32_t batch, float *__restrict__ partial) {
+           float *__restrict__ Y, uint32_t batch, uint32_t spb, float *__restrict__ partial) {
   __shared__ float sW2[MH][MH + 1];  // bf(W2), padded
+  __shared__ float sw3[MH];
   __shared__ float sx[MI], sh1[MH], sh2[MH], sda2[MH];
   __shared__ float sred[2];
   const int i = threadIdx.x;
@@ -39,12 +49,10 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
 #pragma unroll
   for (int j = 0; j < MI; j++) w1[j] = bf(P[OFF_W1 + i * MI + j]);
 #pragma unroll
-  for (int j = 0; j < MH; j++) {
-    w2[j] = bf(P[OFF_W2 + i * MH + j]);
-    sW2[i][j] = w2[j];
-  }
+  for (int j = 0; j < MH; j++) sW2[j][i] = bf(P[OFF_W2 + j * MH + i]);  // coalesced
   const float b1 = bf(P[OFF_B1 + i]), b2 = bf(P[OFF_B2 + i]), w3 = bf(P[OFF_W3 + i]);
   const float b3 = bf(P[OFF_B3]);
+  sw3[i] = w3;
   float gW1[MI], gW2[MH], gb1 = 0.f, gb2 = 0.f, gw3 = 0.f, gb3 = 0.f, loss = 0.f;
   if (BACKWARD) {
 #pragma unroll
@@ -53,8 +61,10 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
     for (int j = 0; j < MH; j++) gW2[j] = 0.f;
   }
   __syncthreads();
-  const uint32_t s0 = blockIdx.x * MLP_SPB;
-  for (uint32_t s = s0; s < s0 + MLP_SPB && s < batch; s++) {
+#pragma unroll
+  for (int j = 0; j < MH; j++) w2[j] = sW2[i][j];
+  const uint32_t s0 = blockIdx.x * spb;
+  for (uint32_t s = s0; s < s0 + spb && s < batch; s++) {
     if (i < MI) sx[i] = bf(X[(size_t)s * MI + i]);
     __syncthreads();
     float a1 = 0.f;
@@ -71,7 +81,8 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
     __syncthreads();
     if (i == 0) {
       float y = 0.f;
-      for (int j = 0; j < MH; j++) y = fmaf(bf(P[OFF_W3 + j]), sh2[j], y);
+#pragma unroll
+      for (int j = 0; j < MH; j++) y = fmaf(sw3[j], sh2[j], y);
       y += b3;
       sred[0] = y;
       if (Y) Y[s] = y;
@@ -90,6 +101,7 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
       for (int j = 0; j < MH; j++) gW2[j] = fmaf(da2, sh1[j], gW2[j]);
       __syncthreads();
       float dh1 = 0.f;
+#pragma unroll 16
       for (int r = 0; r < MH; r++) dh1 = fmaf(sW2[r][i], sda2[r], dh1);
       const float da1 = (a1 > 0.f) ? dh1 : 0.f;
       gb1 += da1;
@@ -100,27 +112,41 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
   }
   if (BACKWARD) {
     float *o = partial + (size_t)blockIdx.x * (N_PARAMS + 1);
+    // W2's gradient goes out through shared memory, a row at a time
+#pragma unroll
+    for (int j = 0; j < MH; j++) sW2[i][j] = gW2[j];
 #pragma unroll
     for (int j = 0; j < MI; j++) o[OFF_W1 + i * MI + j] = gW1[j];
     o[OFF_B1 + i] = gb1;
-#pragma unroll
-    for (int j = 0; j < MH; j++) o[OFF_W2 + i * MH + j] = gW2[j];
     o[OFF_B2 + i] = gb2;
     o[OFF_W3 + i] = gw3;
     if (i == 0) {
       o[OFF_B3] = gb3;
       o[N_PARAMS] = loss;
     }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < MH; j++) o[OFF_W2 + j * MH + i] = sW2[j][i];
   }
 }
 
-// grad[p] = sum over CTAs (in order) of partial[c][p]; loss likewise / batch
-__global__ void mlp_reduce_kernel(const float *__restrict__ partial, uint32_t n_cta, uint32_t batch,
-                                  float *grad, float *loss) {
-  const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p > (uint32_t)N_PARAMS) return;
+// grad[p] = sum over CTAs of partial[c][p], loss likewise / batch: slices of
+// the CTAs in order, then the slices in order
+constexpr int RED_P = 32, RED_S = 16;  // parameters and slices per CTA
+__global__ void __launch_bounds__(RED_P * RED_S)
+mlp_reduce_kernel(const float *__restrict__ partial, uint32_t n_cta, uint32_t batch, float *grad, float *loss) {
+  __shared__ float red[RED_S][RED_P];
+  const uint32_t l = threadIdx.x % RED_P, z = threadIdx.x / RED_P, p = blockIdx.x * RED_P + l;
+  const uint32_t per = (n_cta + RED_S - 1) / RED_S, c1 = min(n_cta, (z + 1) * per);
   float s = 0.f;
-  for (uint32_t c = 0; c < n_cta; c++) s += partial[(size_t)c * (N_PARAMS + 1) + p];
+  if (p <= (uint32_t)N_PARAMS) {
+#pragma unroll 8
+    for (uint32_t c = z * per; c < c1; c++) s += partial[(size_t)c * (N_PARAMS + 1) + p];
+  }
+  red[z][l] = s;
+  __syncthreads();
+  if (z != 0 || p > (uint32_t)N_PARAMS) return;
+  for (int k = 1; k < RED_S; k++) s += red[k][l];
   if (p < (uint32_t)N_PARAMS) grad[p] = s;
   else if (loss) *loss = s / (float)batch;
 }
@@ -137,24 +163,21 @@ __global__ void mlp_adam_kernel(float *p, const float *g, float *m, float *v, ui
   p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-size_t mlp_scratch_floats(uint32_t batch) {
-  const uint32_t n_cta = (batch + MLP_SPB - 1) / MLP_SPB;
-  return (size_t)n_cta * (N_PARAMS + 1);
-}
+size_t mlp_scratch_floats(uint32_t batch) { return (size_t)mlp_ctas(batch) * (N_PARAMS + 1); }
 
 void launch_mlp_forward(const float *params, const float *x, float *y, uint32_t batch, void *stream) {
   if (batch == 0) return;
-  const uint32_t n_cta = (batch + MLP_SPB - 1) / MLP_SPB;
-  mlp_kernel<false><<<n_cta, MH, 0, (cudaStream_t)stream>>>(params, x, nullptr, y, batch, nullptr);
+  mlp_kernel<false><<<mlp_ctas(batch), MH, 0, (cudaStream_t)stream>>>(params, x, nullptr, y, batch, mlp_spb(batch),
+                                                                      nullptr);
 }
 
 void launch_mlp_loss_grad(const float *params, const float *x, const float *target, uint32_t batch,
                           float *loss, float *grad, float *scratch, void *stream) {
   if (batch == 0) return;
-  const uint32_t n_cta = (batch + MLP_SPB - 1) / MLP_SPB;
   cudaStream_t s = (cudaStream_t)stream;
-  mlp_kernel<true><<<n_cta, MH, 0, s>>>(params, x, target, nullptr, batch, scratch);
-  mlp_reduce_kernel<<<(N_PARAMS + 1 + 255) / 256, 256, 0, s>>>(scratch, n_cta, batch, grad, loss);
+  const uint32_t n_cta = mlp_ctas(batch);
+  mlp_kernel<true><<<n_cta, MH, 0, s>>>(params, x, target, nullptr, batch, mlp_spb(batch), scratch);
+  mlp_reduce_kernel<<<(N_PARAMS + RED_P) / RED_P, RED_P * RED_S, 0, s>>>(scratch, n_cta, batch, grad, loss);
 }
 
 void launch_mlp_adam(float *params, const float *grad, float *m, float *v, uint32_t n, uint32_t t,
