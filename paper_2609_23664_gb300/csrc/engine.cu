@@ -88,6 +88,7 @@ struct SvTableBuilder {
   std::vector<SvOpDesc<float>> ops32;
   std::vector<float> ops32lo;  // m[t] - (float)m[t] per FP32 op (compensated passes)
   std::vector<float> ph;       // blocks of the compensated rotation stages (see SvStageDesc::ph_block)
+  std::vector<double> ph64;    // and of FP64 ones
   std::vector<SvOpDesc<double>> ops64;
   bool fp64;
   explicit SvTableBuilder(bool f) : fp64(f) {}
@@ -248,7 +249,7 @@ struct SvTableBuilder {
             }
         }
         sd.rp_mask = rp_stage ? rp_mask : 0u;
-        // a compensated stage of rotations: each real orthogonal 2x2
+        // a compensated or FP64 stage of rotations: each real orthogonal 2x2
         // {r00, r01; r10, r11} is diag(r00, r11) {1, r01/r00; r10/r11, 1};
         // where |r01| is the larger entry the columns are exchanged first
         // (the group is read with that position's halves exchanged), so the
@@ -258,12 +259,12 @@ struct SvTableBuilder {
         // and stored as FP32 pairs
         sd.ph_block = 0xFFFFFFFFu;
         const bool gfold = hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0;
-        if (gfold && (fp64 || pr.g != 4 || !rp_stage)) fail(QW_ERR_STATE, "internal: a global phase on a stage without a table");
-        if (!fp64 && pr.g == 4 && rp_stage) {
-          sd.ph_block = (uint32_t)(ph.size() / SV_PH_BLOCK);
-          float t[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-          double gin[4] = {1, 1, 1, 1};  // input factor of the position's |1> half
-          std::complex<double> d[4][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}};
+        if (gfold && (!rp_stage || (!fp64 && pr.g != 4))) fail(QW_ERR_STATE, "internal: a global phase on a stage without a table");
+        if (rp_stage && (fp64 || pr.g == 4)) {
+          sd.ph_block = (uint32_t)(fp64 ? ph64.size() / (2 * SV_PH64_BLOCK) : ph.size() / SV_PH_BLOCK);
+          double t[SV_G][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
+          double gin[SV_G] = {1, 1, 1, 1, 1};  // input factor of the position's |1> half
+          std::complex<double> d[SV_G][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}, {1, 1}};
           for (const HostOp &o : sops) {
             double r00 = o.m[0], r01 = o.m[1], r10 = o.m[2], r11 = o.m[3];
             if (std::fabs(r01) > std::fabs(r00)) {
@@ -271,24 +272,41 @@ struct SvTableBuilder {
               std::swap(r10, r11);
               sd.ld_xor ^= sd.roff[o.a];
             }
-            const double a1 = exact_rotation(r01 / r00, t[o.a]);
+            double a1 = 1.0;
+            t[o.a][0] = r01 / r00;
+            t[o.a][1] = r10 / r11;
+            if (!fp64) {
+              float T[2];
+              a1 = exact_rotation(r01 / r00, T);
+              t[o.a][0] = T[0];
+              t[o.a][1] = T[1];
+            }
             gin[o.a] = 1.0 / a1;
             d[o.a][0] = r00;
             d[o.a][1] = r11 * a1 * std::complex<double>(o.m[4], o.m[5]);
           }
-          for (uint32_t e = 0; e < 16; e++) {
-            double f = 1.0;
-            for (uint32_t p4 = 0; p4 < 4; p4++)
-              if ((e >> p4) & 1u) f *= gin[p4];
-            ph.push_back((float)(f - 1.0));
-          }
-          for (int p4 = 0; p4 < 4; p4++) ph.insert(ph.end(), {t[p4][0], t[p4][1]});
-          for (uint32_t e = 0; e < 16; e++) {
+          if (!fp64)
+            for (uint32_t e = 0; e < 16; e++) {
+              double f = 1.0;
+              for (uint32_t p4 = 0; p4 < 4; p4++)
+                if ((e >> p4) & 1u) f *= gin[p4];
+              ph.push_back((float)(f - 1.0));
+            }
+          for (uint32_t q = 0; q < pr.g; q++)
+            for (const double v : t[q]) {
+              if (fp64) ph64.push_back(v);
+              else ph.push_back((float)v);
+            }
+          for (uint32_t e = 0; e < (1u << pr.g); e++) {
             std::complex<double> q(hs.gphase[0], hs.gphase[1]);
-            for (uint32_t p4 = 0; p4 < 4; p4++) q *= d[p4][(e >> p4) & 1u];
+            for (uint32_t i = 0; i < pr.g; i++) q *= d[i][(e >> i) & 1u];
             for (const double v : {q.real(), q.imag()}) {
-              ph.push_back((float)v);
-              ph.push_back((float)(v - (double)(float)v));
+              if (fp64) {
+                ph64.push_back(v);
+              } else {
+                ph.push_back((float)v);
+                ph.push_back((float)(v - (double)(float)v));
+              }
             }
           }
           sops.clear();  // the stage runs from its block alone
@@ -630,6 +648,7 @@ static void prepare(qw_plan *P) {
   D->t64.passes = D->arena.upload(b64.passes, s);
   D->t64.stages = D->arena.upload(b64.stages, s);
   D->t64.ops = D->arena.upload(b64.ops64, s);
+  D->t64.ph = D->arena.upload(b64.ph64, s);
 
   // boundary store (budget was enforced by the planner)
   D->mat_buf.assign(P->mats.size(), nullptr);
@@ -1844,7 +1863,7 @@ TileConfig Engine::tile_config(uint32_t n_eff, bool fp64, int ar, uint32_t mix) 
       if (tc.b + 2 > tc.k_max || tc.k_max > best_cap) continue;
       float tot = 0;
       for (const auto &g : circuits) {
-        SvProgram pr = fuse_sv(g.data(), g.size(), key_n, tc);
+        SvProgram pr = fuse_sv(g.data(), g.size(), key_n, tc, fp64);
         SvTableBuilder tb(fp64);
         tb.add(pr);
         SvTables T;
@@ -1853,7 +1872,7 @@ TileConfig Engine::tile_config(uint32_t n_eff, bool fp64, int ar, uint32_t mix) 
         T.stages = dar.upload(tb.stages, s);
         T.ops = fp64 ? (const void *)dar.upload(tb.ops64, s) : (const void *)dar.upload(tb.ops32, s);
         T.ops_lo = fp64 ? nullptr : dar.upload(tb.ops32lo, s);
-        T.ph = fp64 ? nullptr : dar.upload(tb.ph, s);
+        T.ph = fp64 ? (const void *)dar.upload(tb.ph64, s) : (const void *)dar.upload(tb.ph, s);
         // timed in the persistent batch kernel that runs the suffixes: each
         // state's passes a chain of jobs (each waiting for the last), the
         // chains interleaved pass by pass
@@ -1910,7 +1929,7 @@ TileConfig Engine::tile_config(uint32_t n_eff, bool fp64, int ar, uint32_t mix) 
     float tot = 0;
     size_t n_passes = 0;
     for (const auto &g : circuits) {
-      SvProgram pr = fuse_sv(g.data(), g.size(), key_n, best);
+      SvProgram pr = fuse_sv(g.data(), g.size(), key_n, best, fp64);
       SvTableBuilder tb(fp64);
       tb.add(pr);
       SvTables T;
@@ -1919,7 +1938,7 @@ TileConfig Engine::tile_config(uint32_t n_eff, bool fp64, int ar, uint32_t mix) 
       T.stages = dar.upload(tb.stages, s);
       T.ops = fp64 ? (const void *)dar.upload(tb.ops64, s) : (const void *)dar.upload(tb.ops32, s);
       T.ops_lo = fp64 ? nullptr : dar.upload(tb.ops32lo, s);
-      T.ph = fp64 ? nullptr : dar.upload(tb.ph, s);
+      T.ph = fp64 ? (const void *)dar.upload(tb.ph64, s) : (const void *)dar.upload(tb.ph, s);
       for (int r = 0; r < 3; r++) {  // one warm-up, two timed
         cudaEventRecord(e0, s);
         for (size_t p = 0; p < pr.passes.size(); p++)
@@ -2092,7 +2111,7 @@ void costmodel_probe(Engine *E, const Workload &W, float *feat, float *tgt, floa
     for (auto sg : segs) {
       if (rows >= cap || sg.second <= sg.first) continue;
       T.copy_gates(sg.first, sg.second, buf);
-      SvProgram pr = fuse_sv(buf.data(), buf.size(), n_eff, tc);
+      SvProgram pr = fuse_sv(buf.data(), buf.size(), n_eff, tc, fp64);
       SvTableBuilder tb(fp64);
       tb.add(pr);
       DevArena ar;
@@ -2101,7 +2120,7 @@ void costmodel_probe(Engine *E, const Workload &W, float *feat, float *tgt, floa
       Tt.stages = ar.upload(tb.stages, s);
       Tt.ops = fp64 ? (const void *)ar.upload(tb.ops64, s) : (const void *)ar.upload(tb.ops32, s);
       Tt.ops_lo = fp64 ? nullptr : ar.upload(tb.ops32lo, s);
-      Tt.ph = fp64 ? nullptr : ar.upload(tb.ph, s);
+      Tt.ph = fp64 ? (const void *)ar.upload(tb.ph64, s) : (const void *)ar.upload(tb.ph, s);
       float best = 1e30f;
       for (int r = 0; r < 3; r++) {
         cudaEventRecord(e0, s);
@@ -2179,7 +2198,7 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   for (uint64_t i = 0; i < n_gates; i++) n2 += is_two_qubit_op(gates[i].op) ? 1 : 0;
   TileConfig tc = E->tile_config(n, fp64, SV_AR_COMP, gate_mix(n2, n_gates));
   tc.k_max = std::min<uint32_t>(tc.k_max, sv_max_tile(ar, fp64));
-  SvProgram pr = fuse_sv(gates, n_gates, n, tc);
+  SvProgram pr = fuse_sv(gates, n_gates, n, tc, fp64);
   if (pr.passes.empty()) {
     if (!init) return QW_OK;
     HostPass hp;
@@ -2193,7 +2212,7 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   SvTables T;
   Blob bl;
   const size_t op = bl.add(tb.passes), os = bl.add(tb.stages), oo = fp64 ? bl.add(tb.ops64) : bl.add(tb.ops32);
-  const size_t ol = bl.add(tb.ops32lo), oh = bl.add(tb.ph);
+  const size_t ol = bl.add(tb.ops32lo), oh = fp64 ? bl.add(tb.ph64) : bl.add(tb.ph);
   const size_t np = pr.passes.size();
   const size_t tab_bytes = (bl.bytes.size() + 255) & ~(size_t)255;
   const bool keep_rem = ar == SV_AR_REM && np > 1;
@@ -2203,7 +2222,7 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   T.stages = (const SvStageDesc *)(ws.p + os);
   T.ops = ws.p + oo;
   T.ops_lo = (const float *)(ws.p + ol);
-  T.ph = (const float *)(ws.p + oh);
+  T.ph = ws.p + oh;
   void *rem = keep_rem ? ws.p + tab_bytes : nullptr;
   for (size_t p = 0; p < np; p++)
     launch_sv_pass(fp64, T, (uint32_t)p, (uint32_t)pr.passes[p].q.size(), n,

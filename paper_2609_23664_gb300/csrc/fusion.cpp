@@ -212,7 +212,7 @@ static void mat_mul(const double a[8], const double b[8], double out[8]) {  // o
   for (int i = 0; i < 4; i++) { out[2 * i] = C[i].real(); out[2 * i + 1] = C[i].imag(); }
 }
 
-SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const TileConfig &tc) {
+SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const TileConfig &tc, bool fp64) {
   SvProgram prog;
   prog.n = n_eff;
   prog.n_gates = n_gates;
@@ -397,10 +397,10 @@ SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const 
   // fold the global phase into one single-qubit op (every amplitude is in
   // exactly one of its pairs): the first general op if there is one, else
   // the first single-qubit op of any kind
-  // (compensated programs, stages of four positions: carried by the first
+  // (compensated and FP64 programs: carried by the first
   // stage of rotations, whose table multiplies every amplitude anyway, so
   // that its ops stay rotations)
-  if (gphase != cd(1.0, 0.0) && G == (uint32_t)SV_G_COMP && SV_G_PLAIN32 != SV_G_COMP) {
+  if (gphase != cd(1.0, 0.0) && (fp64 || (G == (uint32_t)SV_G_COMP && SV_G_PLAIN32 != SV_G_COMP))) {
     for (auto &ps : prog.passes)
       for (auto &st : ps.stages) {
         if (gphase == cd(1.0, 0.0)) continue;

@@ -1032,7 +1032,7 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
     } else {
       R.copy_gates(M.begin, M.end, buf);
       TileConfig tc = C.tiles(M.n_eff, M.mode == QW_MODE_SV_FP64, true);
-      M.sv = fuse_sv(buf.data(), buf.size(), M.n_eff, tc);
+      M.sv = fuse_sv(buf.data(), buf.size(), M.n_eff, tc, M.mode == QW_MODE_SV_FP64);
       if (P->opts.dense_boundaries) M.gates = buf;
     }
   }
@@ -1046,7 +1046,7 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
     } else {
       T.copy_gates(tp.begin, T.n_gates, buf);
       TileConfig tc = C.tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
-      tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc);
+      tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc, T.mode == QW_MODE_SV_FP64);
       tp.chain = T.mode == QW_MODE_SV_FP32 && plan_ar_batch(P) == SV_AR_COMP &&
                  (!P->opts.batched || tp.sv.passes.size() > (size_t)SV_COMP_MAX_BATCH_PASSES);
       if (tp.chain) {

@@ -133,7 +133,7 @@ struct HostStage {
   uint32_t ctl_w[SV_MAX_OUT_CTL] = {0, 0, 0, 0};  // per-tile terms of c (pass's ctl_q)
   std::vector<HostOp> ops;
   // global phase the stage applies to every amplitude (the first rotation
-  // stage of a compensated program carries the program's, in its table)
+  // stage of a compensated or FP64 program carries the program's, in its table)
   double gphase[2] = {1.0, 0.0};
   HostStage() { for (uint32_t t = 0; t < 32; t++) mcol[t] = 1u << t; }
 };
@@ -198,6 +198,7 @@ struct SvPassDesc {
   uint32_t ctl_tb[SV_MAX_OUT_CTL], ctl_w[SV_MAX_OUT_CTL];
 };
 constexpr uint32_t SV_PH_BLOCK = 16 + 4 * 2 + 16 * 4;  // floats of a rotation stage's block
+constexpr uint32_t SV_PH64_BLOCK = 5 + 32;
 struct alignas(16) SvStageDesc {
   uint32_t roff[SV_G];           // byte offset of phi(e_pos[j]) for register bit j
   uint32_t gcol[SV_MAX_GBITS];   // byte offsets of the group bits (zero past the tile's)
@@ -213,8 +214,10 @@ struct alignas(16) SvStageDesc {
   // remainder, im, im remainder} of the factor it takes after the rotations:
   // the diagonal entries taken out of them, the |1>-phases of e's set
   // positions and the program's global phase where this stage carries it
+  // (FP64 stages of rotations: blocks of SV_PH64_BLOCK double2, the
+  // rotations of the five positions, then the 32 factors)
   uint32_t ph_block;
-  // compensated FP32 stage of rotations: XOR of the roff of the positions
+  // stages of rotations with a block: XOR of the roff of the positions
   // whose two halves are exchanged when the group is read, so that the
   // larger entry of the rotation's rows is on the diagonal
   uint32_t ld_xor;
@@ -230,7 +233,8 @@ struct alignas(16) SvOpDesc {
 static_assert(sizeof(SvOpDesc<float>) == 48 && sizeof(SvOpDesc<double>) == 80, "op descriptor layout");
 
 // Fusion planner: gates -> passes -> stages (host).
-SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const TileConfig &tc);
+// (fp64: for FP64 passes, whose first rotation stage can carry the global phase)
+SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const TileConfig &tc, bool fp64 = false);
 // Number of passes a segment would take (cheap estimate used by the planner).
 uint32_t estimate_passes(uint64_t n_gates, uint32_t n, const TileConfig &tc, double gates_per_pass);
 // Gate matrix in double precision (host). Returns false for non-1q ops.
@@ -390,9 +394,9 @@ struct SvTables {
   const SvStageDesc *stages = nullptr;
   const void *ops = nullptr;       // SvOpDesc<T>*
   const float *ops_lo = nullptr;   // FP32: m[t] - (float)m[t] of every op, 8 floats per op (compensated passes)
-  // compensated FP32: rotations and factors of the rotation stages, blocks
-  // of SV_PH_BLOCK floats (see SvStageDesc::ph_block)
-  const float *ph = nullptr;
+  // rotations and factors of the rotation stages of compensated FP32 and of
+  // FP64 passes (see SvStageDesc::ph_block)
+  const void *ph = nullptr;
 };
 // Arithmetic of FP32 statevector passes.  PLAIN: FP32 registers.  COMP:
 // double-float registers (every op exact to about 2^-48), the amplitude

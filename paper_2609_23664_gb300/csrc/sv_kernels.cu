@@ -144,6 +144,21 @@ __device__ __forceinline__ void op_rp(C (&a)[N], const T (&m)[8]) {
   }
 }
 
+// unnormalized rotation: x' = x + t0 y, y' = y + t1 x
+template <typename C, typename T, int P, int N>
+__device__ __forceinline__ void op_rot(C (&a)[N], const C t) {
+#pragma unroll
+  for (int i = 0; i < N; i++) {
+    if (i & (1 << P)) continue;
+    const int j = i | (1 << P);
+    const C x = a[i], y = a[j];
+    a[i].x = fma(t.x, y.x, x.x);
+    a[i].y = fma(t.x, y.y, x.y);
+    a[j].x = fma(t.y, x.x, y.x);
+    a[j].y = fma(t.y, x.y, y.y);
+  }
+}
+
 // [[c, -is], [-is, c]] with c = m0, s = m1
 template <typename C, typename T, int P, int N>
 __device__ __forceinline__ void op_rx(C (&a)[N], const T (&m)[8]) {
@@ -360,7 +375,7 @@ __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t
 template <typename T, int AR, int G>
 __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__restrict__ stages,
                         const SvOpDesc<T> *__restrict__ ops, const float *__restrict__ ops_lo,
-                        const float *__restrict__ ph,
+                        const void *__restrict__ ph,
                         typename V2<T>::t *sm, const typename V2<T>::t *src, typename V2<T>::t *dst,
                         const float2 *src_lo, float2 *dst_lo, uint32_t tile) {
   typedef typename V2<T>::t C;
@@ -453,18 +468,38 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
 #pragma unroll
       for (int t = 0; t < SV_MAX_GBITS; t++) sbB ^= ((grp >> t) & 1u) ? gcol[t] : 0u;
       if constexpr (AR != SV_AR_PLAIN) {
-        sv_stage_df<AR, G>(smw, lo_off, sbB, sbB ^ ld_xor, roff, ops, ops_lo, op_begin, nops, rp_mask, ph, ph_block);
+        sv_stage_df<AR, G>(smw, lo_off, sbB, sbB ^ ld_xor, roff, ops, ops_lo, op_begin, nops, rp_mask, (const float *)ph, ph_block);
       } else {
       constexpr int N = 1 << G;
+      const uint32_t ldB = sizeof(T) == 8 ? sbB ^ ld_xor : sbB;
       C a[N];
 #pragma unroll
       for (int i = 0; i < N; i++) {
-        const uint32_t off = sbB ^ ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^
+        const uint32_t off = ldB ^ ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^
                              ((i & 4) ? roff[2] : 0u) ^ ((i & 8) ? roff[3] : 0u) ^
                              ((G > 4 && (i & 16)) ? roff[4] : 0u);
         a[i] = *(const C *)(smc + off);
       }
-      if (rp_mask) {
+      if (sizeof(T) == 8 && rp_mask) {
+        // FP64 rotations on distinct positions: unnormalized, two FMAs per
+        // amplitude, then one factor per amplitude (their diagonals, phases
+        // and the program's global phase).  The FP64 pipe (1/64 of the FP32
+        // rate) bounds these passes: 448 FP64 operations per 32 amplitudes
+        // and full stage instead of 960
+        const C *blk = (const C *)ph + SV_PH64_BLOCK * (size_t)ph_block;
+        if (rp_mask & 1u) op_rot<C, T, 0, N>(a, __ldg(blk));
+        if (rp_mask & 2u) op_rot<C, T, 1, N>(a, __ldg(blk + 1));
+        if (rp_mask & 4u) op_rot<C, T, 2, N>(a, __ldg(blk + 2));
+        if (rp_mask & 8u) op_rot<C, T, 3, N>(a, __ldg(blk + 3));
+        if constexpr (G > 4)
+          if (rp_mask & 16u) op_rot<C, T, 4, N>(a, __ldg(blk + 4));
+#pragma unroll
+        for (int i = 0; i < N; i++) {
+          const C w = __ldg(blk + SV_G + i), x = a[i];
+          a[i].x = w.x * x.x - w.y * x.y;
+          a[i].y = w.x * x.y + w.y * x.x;
+        }
+      } else if (rp_mask) {
         // rotation-and-phase ops on distinct positions, in position order
         const SvOpDesc<T> *op = ops + op_begin;
 #pragma unroll
