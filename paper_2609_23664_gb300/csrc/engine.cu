@@ -261,7 +261,7 @@ struct SvTableBuilder {
         const bool gfold = hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0;
         if (gfold && (!rp_stage || (!fp64 && pr.g != 4))) fail(QW_ERR_STATE, "internal: a global phase on a stage without a table");
         if (rp_stage && (fp64 || pr.g == 4)) {
-          sd.ph_block = (uint32_t)(fp64 ? ph64.size() / (2 * SV_PH64_BLOCK) : ph.size() / SV_PH_BLOCK);
+          sd.ph_block = fp64 ? (uint32_t)(ph64.size() / (2 * SV_PH64_BLOCK)) : (uint32_t)stages.size();
           double t[SV_G][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
           double gin[SV_G] = {1, 1, 1, 1, 1};  // input factor of the position's |1> half
           std::complex<double> d[SV_G][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}, {1, 1}};
@@ -334,6 +334,9 @@ struct SvTableBuilder {
           }
         }
         stages.push_back(sd);
+        // compensated programs have a block per stage (zero where unused), so
+        // that a stage's descriptor and block are fetched together
+        if (!fp64 && pr.g == 4) ph.resize(stages.size() * SV_PH_BLOCK, 0.f);
       }
       passes.push_back(d);
     }

@@ -208,7 +208,7 @@ struct alignas(16) SvStageDesc {
   // one per position in ascending order (run without dispatch)
   uint32_t rp_mask;
   // compensated FP32 stage of rotations: block of SV_PH_BLOCK floats of the
-  // table array: for each amplitude index e of the group the input factor
+  // table array (the stage's own index): for each amplitude index e of the group the input factor
   // less one (16), the unnormalized rotation {t0, t1} of each of the four
   // positions (zero where the mask has none), then for each e {re, re
   // remainder, im, im remainder} of the factor it takes after the rotations:

@@ -273,7 +273,7 @@ template <int AR, int G>
 __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t sbB, uint32_t ldB,
                                             const uint32_t (&roff)[SV_G], const SvOpDesc<float> *__restrict__ ops,
                                             const float *__restrict__ ops_lo, uint32_t op_begin, uint32_t nops,
-                                            uint32_t rp_mask, const float *__restrict__ ph, uint32_t ph_block) {
+                                            uint32_t rp_mask, const float *blk) {
   constexpr int N = 1 << G;
   static_assert(G == 4, "the phase block holds four rotations and 16 entries");
   auto off = [&](int i) {
@@ -307,32 +307,31 @@ __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t
     l[i] = r;
   };
   if (rp_mask) {
-    const float *blk = ph + SV_PH_BLOCK * (size_t)ph_block;
     const float2 *t = (const float2 *)(blk + 16);
     if (rp_mask == 0xFu) {
-      const float2 t0 = __ldg(t);
+      const float2 t0 = t[0];
 #pragma unroll
       for (int i = 0; i < N; i += 2) {
-        const float2 e = __ldg((const float2 *)(blk + i));
+        const float2 e = *(const float2 *)(blk + i);
         split(i, e.x);
         split(i + 1, e.y);
         gd_pair(C, t0, H[i], l[i], H[i + 1], l[i + 1]);
       }
-      gdop_rot<1, N>(C, H, l, __ldg(t + 1));
-      gdop_rot<2, N>(C, H, l, __ldg(t + 2));
-      gdop_rot<3, N>(C, H, l, __ldg(t + 3));
+      gdop_rot<1, N>(C, H, l, t[1]);
+      gdop_rot<2, N>(C, H, l, t[2]);
+      gdop_rot<3, N>(C, H, l, t[3]);
     } else {
 #pragma unroll
-      for (int i = 0; i < N; i++) split(i, __ldg(blk + i));
-      if (rp_mask & 1u) gdop_rot<0, N>(C, H, l, __ldg(t));
-      if (rp_mask & 2u) gdop_rot<1, N>(C, H, l, __ldg(t + 1));
-      if (rp_mask & 4u) gdop_rot<2, N>(C, H, l, __ldg(t + 2));
-      if (rp_mask & 8u) gdop_rot<3, N>(C, H, l, __ldg(t + 3));
+      for (int i = 0; i < N; i++) split(i, blk[i]);
+      if (rp_mask & 1u) gdop_rot<0, N>(C, H, l, t[0]);
+      if (rp_mask & 2u) gdop_rot<1, N>(C, H, l, t[1]);
+      if (rp_mask & 4u) gdop_rot<2, N>(C, H, l, t[2]);
+      if (rp_mask & 8u) gdop_rot<3, N>(C, H, l, t[3]);
     }
     const float4 *q = (const float4 *)(blk + 24);
 #pragma unroll
     for (int e = 0; e < N; e++) {
-      const float4 w = __ldg(q + e);
+      const float4 w = q[e];
       gd_cmul(C, w.x, w.y, w.z, w.w, H[e], l[e]);
     }
   } else {
@@ -409,6 +408,20 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
     gstep[t] = lb < k ? gdep(1u << lb) : 0u;
     sstep[t] = lb < k ? swz<T>(1u << lb) * (uint32_t)sizeof(C) : 0u;
   }
+  // Compensated passes: a stage's descriptor and table (29 16-byte words) are
+  // copied to shared memory while the previous stage runs
+  constexpr uint32_t SD = sizeof(SvStageDesc) / 16, SB = SV_PH_BLOCK / 4;
+  __shared__ uint4 staged[AR != SV_AR_PLAIN ? 2 : 1][AR != SV_AR_PLAIN ? SD + SB : 1];
+  auto fetch_stage = [&](uint32_t s) {
+    if constexpr (AR != SV_AR_PLAIN) {
+      const size_t at = (size_t)pd->stage_begin + s;
+      if (threadIdx.x < SD)
+        cp_async16(&staged[s & 1][threadIdx.x], (const uint4 *)(stages + at) + threadIdx.x);
+      else if (threadIdx.x < SD + SB)
+        cp_async16(&staged[s & 1][threadIdx.x], (const uint4 *)ph + SB * at + (threadIdx.x - SD));
+    }
+  };
+  if (pd->n_stages) fetch_stage(0);
   const uint32_t l0 = threadIdx.x * APU;
   const char *smc = (const char *)sm;
   char *smw = (char *)sm;
@@ -438,6 +451,7 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
       sm[swz<T>(l)] = v;
       if constexpr (AR == SV_AR_REM) *(float2 *)(smw + lo_off + swz<T>(l) * (uint32_t)sizeof(C)) = make_float2(0.f, 0.f);
     }
+    if constexpr (AR != SV_AR_PLAIN) cp_async_wait_all();
   }
   __syncthreads();
 
@@ -449,9 +463,13 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
   const uint32_t n_groups = 1u << (k - G);
   const uint32_t n_st = pd->n_stages, st0 = pd->stage_begin;
   for (uint32_t s = 0; s < n_st; s++) {
-    const uint4 *sdv = (const uint4 *)(stages + st0 + s);
-    const uint4 w0 = __ldg(sdv), w1 = __ldg(sdv + 1), w2 = __ldg(sdv + 2), w3 = __ldg(sdv + 3),
-                w4 = __ldg(sdv + 4), w5 = __ldg(sdv + 5), w6 = __ldg(sdv + 6);
+    const uint4 *sdv = AR != SV_AR_PLAIN ? staged[s & 1] : (const uint4 *)(stages + st0 + s);
+    auto word = [&](int i) {
+      if constexpr (AR != SV_AR_PLAIN) return sdv[i];
+      else return __ldg(sdv + i);
+    };
+    if (AR != SV_AR_PLAIN && s + 1 < n_st) fetch_stage(s + 1);
+    const uint4 w0 = word(0), w1 = word(1), w2 = word(2), w3 = word(3), w4 = word(4), w5 = word(5), w6 = word(6);
     // offsets are masked to the tile, so XOR combinations stay inside it
     const uint32_t tm = ntile * (uint32_t)sizeof(C) - 1u;
     const uint32_t roff[SV_G] = {w0.x & tm, w0.y & tm, w0.z & tm, w0.w & tm, w1.x & tm};
@@ -468,7 +486,8 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
 #pragma unroll
       for (int t = 0; t < SV_MAX_GBITS; t++) sbB ^= ((grp >> t) & 1u) ? gcol[t] : 0u;
       if constexpr (AR != SV_AR_PLAIN) {
-        sv_stage_df<AR, G>(smw, lo_off, sbB, sbB ^ ld_xor, roff, ops, ops_lo, op_begin, nops, rp_mask, (const float *)ph, ph_block);
+        sv_stage_df<AR, G>(smw, lo_off, sbB, sbB ^ ld_xor, roff, ops, ops_lo, op_begin, nops, rp_mask,
+                           (const float *)(staged[s & 1] + SD));
       } else {
       constexpr int N = 1 << G;
       const uint32_t ldB = sizeof(T) == 8 ? sbB ^ ld_xor : sbB;
@@ -535,6 +554,7 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
       }
       }
     }
+    if constexpr (AR != SV_AR_PLAIN) cp_async_wait_all();  // the next stage's data
     __syncthreads();
   }
 
