@@ -875,14 +875,20 @@ static void prepare(qw_plan *P) {
   size_t max_partials = 1, max_smp_blocks = 1, max_src = 1;
   const bool batched = P->opts.batched != 0;
   // Compensated FP32 tasks with long programs keep their remainder between
-  // passes.  Where the tiles of one pass take at most half of the resident
-  // CTAs (up to 19 qubits), several tasks advance together in a persistent
-  // launch, each with its remainder array; larger registers fill the chip
-  // alone and run one after another, pass by pass.
+  // passes.  Where a pass alone leaves much of the chip idle, several tasks
+  // advance together in a persistent launch, each with its remainder array:
+  // where its tiles take at most half of the resident CTAs (up to 19 qubits:
+  // 64 tiles of 18 qubits left 86 % idle), or where they take two or three
+  // rounds of them and the last is less than half full (21 and 22 qubits: 512
+  // and 1024 tiles on 456 CTAs).  Other registers fill the chip alone and run
+  // one task after another, pass by pass.
   auto long_chain = [&](const TaskPlan &tp) { return batched && tp.chain; };
   const uint32_t rem_slots = (uint32_t)sv_batch_grid(false, SV_MAX_TILE_FP32_REM, E->sm_count, SV_AR_REM);
   auto shares_launch = [&](const TaskPlan &tp) {
-    return !tp.sv.passes.empty() && 2u << (tp.n_eff - (uint32_t)tp.sv.passes[0].q.size()) <= rem_slots;
+    if (tp.sv.passes.empty()) return false;
+    const uint64_t tiles = 1ull << (tp.n_eff - (uint32_t)tp.sv.passes[0].q.size());
+    const uint64_t rounds = (tiles + rem_slots - 1) / rem_slots, last = tiles - (rounds - 1) * rem_slots;
+    return 2 * tiles <= rem_slots || ((rounds == 2 || rounds == 3) && 2 * last < rem_slots);
   };
   // Task buffers of every group coexist for the plan's lifetime, so the
   // groups share one task budget: each group with pooled tasks gets one
