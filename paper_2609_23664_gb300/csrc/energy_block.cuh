@@ -133,11 +133,16 @@ __device__ __forceinline__ float en_pairs(const float2 (&a)[EnAmp<float, PAIR>::
       for (int k = 0; k < w; k++) v[k] = fmaf(s[b], v[2 * k + 1], v[2 * k]);
     return v[0];
   } else {
-    float2 v[NP];
+    // the first level takes every second product unrounded: its sign goes
+    // to one factor (exact), the product into the multiply-add
+    float2 v[NP / 2];
 #pragma unroll
-    for (int k = 0; k < NP; k++) v[k] = __fmul2_rn(a[en_low<MC, E, PAIR>(k) ^ m], a[en_low<MC, E, PAIR>(k)]);
+    for (int k = 0; k < NP / 2; k++) {
+      const int i = en_low<MC, E, PAIR>(2 * k), j = en_low<MC, E, PAIR>(2 * k + 1);
+      v[k] = __ffma2_rn(__fmul2_rn(make_float2(s[0], s[0]), a[j ^ m]), a[j], __fmul2_rn(a[i ^ m], a[i]));
+    }
 #pragma unroll
-    for (int w = NP / 2, b = 0; w > 0; w /= 2, b++) {
+    for (int w = NP / 4, b = 1; w > 0; w /= 2, b++) {
       const float2 sb = make_float2(s[b], s[b]);
 #pragma unroll
       for (int k = 0; k < w; k++) v[k] = __ffma2_rn(sb, v[2 * k + 1], v[2 * k]);
@@ -225,7 +230,7 @@ __device__ __forceinline__ void en_pin(double2 (&a)[N]) {
 
 // one term on the basis mask of combination MC
 template <typename T, int MC, bool PAIR, typename C>
-__device__ __forceinline__ void en_slot(const C (&a)[EnAmp<T, PAIR>::N], const EnTerm *t, uint32_t x0, T &e) {
+__device__ __forceinline__ void en_slot(const C (&a)[EnAmp<T, PAIR>::N], const EnTerm *t, uint32_t x0, typename AccOf<T>::t &acc) {
   const uint4 q = __ldg((const uint4 *)t);
   const T coef = en_coef<T>(q);
   const EnSign<T> sg(t, q.y);
@@ -235,13 +240,13 @@ __device__ __forceinline__ void en_slot(const C (&a)[EnAmp<T, PAIR>::N], const E
     if (q.y & 32u) {
       if (q.y & 16u) s = en_pairs<MC, 1, true, PAIR>(a, sg.get());
       else s = en_pairs<MC, 1, false, PAIR>(a, sg.get());
-      e = fma(c, s, e);
+      acc.add(c * s);
       return;
     }
   }
   if (q.y & 16u) s = en_pairs<MC, 0, true, PAIR>(a, sg.get());
   else s = en_pairs<MC, 0, false, PAIR>(a, sg.get());
-  e = fma(c, s, e);
+  acc.add(c * s);
 }
 
 // Block `jb` of energy job J: 2^J.rep_bits coset representatives of each of
@@ -296,30 +301,24 @@ __device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const 
         for (int k = 0; k < N; k++) s += a[k].x * a[k].x + a[k].y * a[k].y;
         nrm += s;
       }
-      T e = 0;
       uint32_t t = w.y;
       // the first terms flip the basis masks, one each: straight-line code, a
       // uniform branch or two each (random Hamiltonians hold few others)
       const uint32_t ns = w.w >> EN_GROUP_SLOTS_SHIFT;
-      if (ns > 0) en_slot<T, 1, PAIR>(a, tab.terms + t, x0, e);
-      if (ns > 1) en_slot<T, 2, PAIR>(a, tab.terms + t + 1, x0, e);
-      if (ns > 2) en_slot<T, 4, PAIR>(a, tab.terms + t + 2, x0, e);
-      if (ns > 3) en_slot<T, 8, PAIR>(a, tab.terms + t + 3, x0, e);
+      if (ns > 0) en_slot<T, 1, PAIR>(a, tab.terms + t, x0, acc);
+      if (ns > 1) en_slot<T, 2, PAIR>(a, tab.terms + t + 1, x0, acc);
+      if (ns > 2) en_slot<T, 4, PAIR>(a, tab.terms + t + 2, x0, acc);
+      if (ns > 3) en_slot<T, 8, PAIR>(a, tab.terms + t + 3, x0, acc);
       t += ns;
 #pragma unroll 1
-      for (uint32_t i = 0; t < w.z; t++, i++) {
-        if ((i & 3u) == 0) {  // at most four terms between two-sums
-          acc.add(e);
-          e = 0;
-        }
+      for (; t < w.z; t++) {
         const uint4 q = __ldg((const uint4 *)(tab.terms + t));  // zm, code, coef
         const T coef = en_coef<T>(q);
         const EnSign<T> sg(tab.terms + t, q.y);
         en_pin(a);
         const T s = en_pairs_rt<T, PAIR>(a, q.y, sg);
-        e = fma((__popc(x0 & q.x) & 1) ? -coef : coef, s, e);
+        acc.add(((__popc(x0 & q.x) & 1) ? -coef : coef) * s);
       }
-      acc.add(e);
     }
   }
   __shared__ double en_red[2][8];

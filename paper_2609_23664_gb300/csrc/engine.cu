@@ -1766,8 +1766,9 @@ void Engine::dev_free(void *p, size_t bytes) {
 }
 
 void Engine::trim_cache() {
-  if (free_blocks.empty()) return;
   cudaSetDevice(device);
+  if (call_pool) cudaMemPoolTrimTo((cudaMemPool_t)call_pool, 0);
+  if (free_blocks.empty()) return;
   cudaDeviceSynchronize();
   for (auto &b : free_blocks) cudaFree(b.second);
   free_blocks.clear();

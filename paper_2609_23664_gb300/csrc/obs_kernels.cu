@@ -167,7 +167,9 @@ EnLayout build_energy_layout(const qw_pauli_term *terms, uint64_t n_terms, uint3
 // registers): 64 24-qubit states, 200 terms: 27.7 ms, against 30.9 ms with
 // four CTAs, 33.6 ms with six (which spill), 31.6 ms with two of 256 threads,
 // 33.1 ms for cosets of 16 amplitudes on 32 warps per SM (bound by
-// instruction issue) and 47 ms term by term.
+// instruction issue) and 47 ms term by term.  A two-sum per term instead of
+// one per group makes it 28.6 ms and the energy of a random state err by
+// 5.3e-8 of its typical size instead of 6.6e-8 (6.5e-8 term by term).
 template <typename T, bool PAIR>
 __global__ void __launch_bounds__(EN_THREADS, sizeof(T) == 8 ? 4 : PAIR ? 5 : 8)
 energy_kernel(EnTables t, uint32_t n_jobs) {
