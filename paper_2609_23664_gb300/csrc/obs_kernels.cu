@@ -283,7 +283,8 @@ __device__ void lane_sums(const typename V2o<T>::t *psi, uint32_t dim, uint32_t 
   int32_t last = -1;
   const uint32_t b0 = off + (uint32_t)ln * SMP_PER_LANE;
   if constexpr (sizeof(T) == 4) {
-    if (b0 + SMP_PER_LANE <= dim) {  // FP32, whole segment: two amplitudes per 16-byte load
+    // FP32, whole segment of a state on a 16-byte boundary: two amplitudes per load
+    if (b0 + SMP_PER_LANE <= dim && ((uintptr_t)psi & 15u) == 0) {
       const float4 *q = reinterpret_cast<const float4 *>(psi + b0);
 #pragma unroll 8
       for (int i = 0; i < SMP_PER_LANE / 2; i++) {
@@ -321,25 +322,88 @@ __device__ __forceinline__ double chain_scan(double s, int ln) {
   return S;
 }
 
+// The lane sums of a whole FP32 block on a 16-byte boundary, read in memory
+// order: 16 amplitudes of every lane's segment at a time (32 lines of 128
+// bytes) are copied to shared memory, eight lanes to a line, two such pieces
+// in flight, and each lane then adds its own row (rows padded to 144 bytes:
+// a quarter warp's 16-byte reads cover every bank).  Each lane reading its
+// segment directly touches 32 lines per load instruction, which the L1 takes
+// one per clock (4.2 TB/s).
+constexpr int SMP_PIECE = 16, SMP_ROW = SMP_PIECE * 8 + 16;  // amplitudes, padded bytes
+struct SmpStage {
+  unsigned char b[2][32 * SMP_ROW];
+};
+__device__ __forceinline__ void smp_fetch(SmpStage &st, const float2 *blk, int piece, int ln) {
+  const uint32_t sm = (uint32_t)__cvta_generic_to_shared(st.b[piece & 1]);
+#pragma unroll
+  for (int u = 0; u < 8; u++) {
+    const int r = u * 4 + (ln >> 3), c = ln & 7;
+    const float2 *g = blk + r * SMP_PER_LANE + piece * SMP_PIECE + 2 * c;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sm + (uint32_t)(r * SMP_ROW + c * 16)), "l"(g)
+                 : "memory");
+  }
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+}
+__device__ __forceinline__ void lane_sums_staged(SmpStage &st, const float2 *blk, int ln, double *lane_sum,
+                                                 int32_t *lane_last) {
+  constexpr int PIECES = SMP_PER_LANE / SMP_PIECE;
+  SmpAcc<float> s;
+  int32_t last = -1;
+  smp_fetch(st, blk, 0, ln);
+#pragma unroll 1
+  for (int p = 0; p < PIECES; p++) {
+    if (p + 1 < PIECES) {
+      smp_fetch(st, blk, p + 1, ln);
+      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    }
+    __syncwarp();
+    const float4 *q = (const float4 *)(st.b[p & 1] + ln * SMP_ROW);
+#pragma unroll
+    for (int i = 0; i < SMP_PIECE / 2; i++) {
+      const float4 v = q[i];
+      const float p0 = fmaf(v.x, v.x, v.y * v.y), p1 = fmaf(v.z, v.z, v.w * v.w);
+      const int at = ln * SMP_PER_LANE + p * SMP_PIECE + 2 * i;
+      s.add(p0);
+      if (p0 > 0) last = at;
+      s.add(p1);
+      if (p1 > 0) last = at + 1;
+    }
+    __syncwarp();  // the piece is overwritten by the fetch after next
+  }
+  *lane_sum = s.value();
+  *lane_last = last;
+}
+
 // One warp per block; the lane sums of the CTA's blocks are chained by one
 // thread per block, all of them at once (the 31 dependent FP64 adds of a
 // chain cost a warp the same for one block as for 32, and at 1/64 of the
 // FP32 rate they showed beside the loads).
-constexpr int SMP_WARPS = 8;
+constexpr int SMP_WARPS = 4;
 template <typename T>
 __global__ void __launch_bounds__(SMP_WARPS * 32)
 smp_blocksum_kernel(const SmpSource *__restrict__ srcs, uint32_t n_src, uint32_t total, double *bsum, int32_t *blast) {
   typedef typename V2o<T>::t C;
   __shared__ double ls[SMP_WARPS][33];
   __shared__ int32_t ll[SMP_WARPS];
+  __shared__ __align__(16) unsigned char stage[sizeof(T) == 4 ? SMP_WARPS * sizeof(SmpStage) : 16];
   const uint32_t w = threadIdx.x / 32, gb = blockIdx.x * SMP_WARPS + w;
   const int ln = threadIdx.x & 31;
   if (gb < total) {
     const SmpSource S = srcs[find_source(srcs, n_src, gb)];
     const uint32_t blk = gb - S.block_begin;
+    const C *psi = (const C *)S.state;
     double s;
     int32_t last;
-    lane_sums<T>((const C *)S.state, 1u << S.n, blk << SMP_BLOCK_BITS, ln, &s, &last);
+    bool done = false;
+    if constexpr (sizeof(T) == 4) {
+      if (S.n >= (uint32_t)SMP_BLOCK_BITS && ((uintptr_t)psi & 15u) == 0) {
+        lane_sums_staged(((SmpStage *)stage)[w], psi + ((size_t)blk << SMP_BLOCK_BITS), ln, &s, &last);
+        done = true;
+      }
+    }
+    if (!done) lane_sums<T>(psi, 1u << S.n, blk << SMP_BLOCK_BITS, ln, &s, &last);
     ls[w][ln] = s;
     last = __reduce_max_sync(0xffffffffu, last);
     if (ln == 0) ll[w] = last;
