@@ -208,7 +208,8 @@ typedef struct qw_plan_opts {
   uint32_t min_group;         /* early filter: tasks sharing a prefix (Sec. IV-A)   */
   uint32_t min_prefix_gates;  /* early filter: prefix length                        */
   double min_prefix_cost_ns;  /* early filter: estimated prefix cost                */
-  uint32_t tile_qubits;       /* 0 = autotuned; else statevector tile size (qubits) */
+  uint32_t tile_qubits;       /* 0 = autotuned; else statevector tile size (qubits; passes that
+                                 keep an FP32 remainder take at most 12) */
   uint32_t low_qubits;        /* 0 = autotuned; contiguous low qubits in every tile */
   uint32_t window;            /* 0 = autotuned; tasks interleaved in the batch order */
   int32_t use_graph;          /* 1 = capture execution in a CUDA graph              */
@@ -258,8 +259,9 @@ typedef struct qw_plan_opts {
                                  FP32 meets).
                                  QW_FP32_COMPENSATED: every amplitude is held
                                  as an unevaluated sum of two FP32 numbers while gates
-                                 run (error-free products and sums on the FP32 units,
-                                 gate constants to 2^-48), so a state is rounded only
+                                 run (an operation errs by about 2^-39 of the largest
+                                 amplitude it works with, rotations by 2^-34 of their
+                                 angle's tangent), so a state is rounded only
                                  when it is stored: the passes of a boundary keep their
                                  FP32 remainder in a second array and round once, into
                                  the boundary; a task's suffix passes round at each

@@ -400,9 +400,9 @@ struct SvTables {
   const void *ph = nullptr;
 };
 // Arithmetic of FP32 statevector passes.  PLAIN: FP32 registers.  COMP:
-// double-float registers (every op exact to about 2^-48), the amplitude
-// rounded to FP32 when its stage writes it back.  REM: double-float
-// through the whole pass (a remainder plane beside the shared-memory tile)
+// two FP32 numbers per component while a stage runs (an op errs by about
+// 2^-39 of its group's largest amplitude), the amplitude rounded to FP32
+// when its stage writes it back.  REM: two numbers through the whole pass (a remainder plane beside the shared-memory tile)
 // and between passes (remainder arrays beside the state), so a chain of
 // passes rounds once, when it writes a state without its remainder.
 enum SvArith : int { SV_AR_PLAIN = 0, SV_AR_COMP = 1, SV_AR_REM = 2 };

@@ -26,7 +26,7 @@
 // rotation output 5 (and one more to un-bias its operand), against 16 for
 // the double-float arithmetic this replaced (products split by FMA, sums by
 // TwoSum): a full rotation stage takes 41 packed instructions per amplitude
-// instead of 80, and the kernels that run it are bound by the FMA pipe.
+// instead of 80 (64-task 24-qubit suffix launch: 104 -> 61 ms), and the kernels that run it are bound by the FMA pipe.
 //
 // Without compensation, the FP32 roundings of the ~600 rotations that every
 // amplitude of a 24-qubit, 24-layer ansatz goes through move a Pauli-sum
