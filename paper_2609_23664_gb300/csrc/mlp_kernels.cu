@@ -28,7 +28,7 @@ static_assert(N_PARAMS == QW_MLP_PARAMS, "parameter layout");
 // the allocator maps at a time.
 constexpr uint32_t MLP_MAX_CTAS = 100;
 static uint32_t mlp_spb(uint32_t batch) { return (batch + MLP_MAX_CTAS - 1) / MLP_MAX_CTAS; }
-static uint32_t mlp_ctas(uint32_t batch) {
+uint32_t mlp_grad_ctas(uint32_t batch) {
   const uint32_t spb = mlp_spb(batch);
   return spb ? (batch + spb - 1) / spb : 0;
 }
@@ -163,11 +163,16 @@ __global__ void mlp_adam_kernel(float *p, const float *g, float *m, float *v, ui
   p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
 }
 
-size_t mlp_scratch_floats(uint32_t batch) { return (size_t)mlp_ctas(batch) * (N_PARAMS + 1); }
+// Covers every batch up to `batch`: training allocates it once and reuses it
+// for the shorter last batch of an epoch, which may take more CTAs than a
+// full one (256 samples take 86, 100 take 100).
+size_t mlp_scratch_floats(uint32_t batch) {
+  return (size_t)(batch < MLP_MAX_CTAS ? batch : MLP_MAX_CTAS) * (N_PARAMS + 1);
+}
 
 void launch_mlp_forward(const float *params, const float *x, float *y, uint32_t batch, void *stream) {
   if (batch == 0) return;
-  mlp_kernel<false><<<mlp_ctas(batch), MH, 0, (cudaStream_t)stream>>>(params, x, nullptr, y, batch, mlp_spb(batch),
+  mlp_kernel<false><<<mlp_grad_ctas(batch), MH, 0, (cudaStream_t)stream>>>(params, x, nullptr, y, batch, mlp_spb(batch),
                                                                       nullptr);
 }
 
@@ -175,7 +180,7 @@ void launch_mlp_loss_grad(const float *params, const float *x, const float *targ
                           float *loss, float *grad, float *scratch, void *stream) {
   if (batch == 0) return;
   cudaStream_t s = (cudaStream_t)stream;
-  const uint32_t n_cta = mlp_ctas(batch);
+  const uint32_t n_cta = mlp_grad_ctas(batch);
   mlp_kernel<true><<<n_cta, MH, 0, s>>>(params, x, target, nullptr, batch, mlp_spb(batch), scratch);
   mlp_reduce_kernel<<<(N_PARAMS + RED_P) / RED_P, RED_P * RED_S, 0, s>>>(scratch, n_cta, batch, grad, loss);
 }

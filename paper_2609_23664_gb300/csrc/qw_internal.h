@@ -555,5 +555,7 @@ void launch_mlp_loss_grad(const float *params, const float *x, const float *targ
                           float *loss, float *grad, float *scratch, void *stream);
 void launch_mlp_adam(float *params, const float *grad, float *m, float *v, uint32_t n, uint32_t t,
                      float lr, float b1, float b2, float eps, void *stream);
+// CTAs (one gradient partial each) of a batch, and the workspace of batches up to this size
+uint32_t mlp_grad_ctas(uint32_t batch);
 size_t mlp_scratch_floats(uint32_t batch);
 }  // namespace qw
