@@ -434,7 +434,7 @@ def run_native(a):
                 "algorithmic_bytes_per_launch": alg}
 
     # the persistent suffix launch: compensated FP32 passes are bound by
-    # FP32 arithmetic (41 packed instructions per amplitude of a full
+    # FP32 arithmetic (44 packed instructions per amplitude of a full
     # rotation stage), plain ones by latency against HBM
     t_sv = batch_flops / (suffix_ms * 1e-3) / 1e12 if suffix_ms > 0 else 0.0
     sv = {"kernel": "sv_batch_kernel", "launch_ms": suffix_ms, "fp32_arith": cr.get("fp32_arith"),

@@ -259,9 +259,10 @@ typedef struct qw_plan_opts {
                                  FP32 meets).
                                  QW_FP32_COMPENSATED: every amplitude is held
                                  as an unevaluated sum of two FP32 numbers while gates
-                                 run (an operation errs by about 2^-39 of the largest
-                                 amplitude it works with, rotations by 2^-34 of their
-                                 angle's tangent), so a state is rounded only
+                                 run (gate constants to 2^-48; an operation errs by about
+                                 2^-39 of the largest of the 16 amplitudes it works with,
+                                 and amplitudes below 2^-15 of that one keep the relative
+                                 precision of plain FP32), so a state is rounded only
                                  when it is stored: the passes of a boundary keep their
                                  FP32 remainder in a second array and round once, into
                                  the boundary; a task's suffix passes round at each

@@ -58,30 +58,6 @@ void launch_copy(const void *src, void *dst, size_t bytes, void *stream) {
 // ---------------------------------------------------------------------------
 // device-side tables of a set of statevector programs
 // ---------------------------------------------------------------------------
-// Writes {1, t; -t, 1} as diag(1, a1) {1, T0; T1, 1} diag(1, 1 / a1) with T0
-// and T1 exact in FP32, and returns a1.  That needs T0 T1 = -t^2: with
-// s t in [2^22, 2^23] for a power of two s, A an integer just above s t and
-// k the integer nearest sqrt(A^2 - (s t)^2), (A + k)(A - k) differs from
-// (s t)^2 by at most k < 2^14, that is 2^-31 of it; the best of eight A is
-// taken (2^-34 typically), a1 = (A + k) / (s t) = 1 + O(2^-10).
-static double exact_rotation(double t, float T[2]) {
-  T[0] = T[1] = 0.f;
-  if (!(std::fabs(t) > 1e-30)) return 1.0;
-  int ex;
-  std::frexp(std::fabs(t), &ex);
-  const double st = std::ldexp(std::fabs(t), 23 - ex), tau = st * st;
-  double A = 0, k = 0, best = 1e300;
-  const double a0 = std::ceil(st);
-  for (int i = 0; i < 8; i++) {
-    const double a = a0 + i, kk = std::nearbyint(std::sqrt(a * a - tau)), r = std::fabs(a * a - kk * kk - tau);
-    if (r < best) { best = r; A = a; k = kk; }
-  }
-  const double unit = std::ldexp(t < 0 ? -1.0 : 1.0, ex - 23);
-  T[0] = (float)((A + k) * unit);
-  T[1] = (float)(-(A - k) * unit);
-  return (A + k) / st;
-}
-
 struct SvTableBuilder {
   std::vector<SvPassDesc> passes;
   std::vector<SvStageDesc> stages;
@@ -255,15 +231,16 @@ struct SvTableBuilder {
         // (the group is read with that position's halves exchanged), so the
         // off-diagonal quotients stay within 1.  The diagonals commute with
         // the other positions' rotations: amplitude e takes their product,
-        // with the |1>-phases of its set positions, computed here in FP64
-        // and stored as FP32 pairs
+        // with the |1>-phases of its set positions.  Quotients and products
+        // are computed here in FP64 and, for compensated stages, stored as
+        // FP32 pairs (to 2^-48: the same angle repeated thousands of times
+        // adds its constants' error up)
         sd.ph_block = 0xFFFFFFFFu;
         const bool gfold = hs.gphase[0] != 1.0 || hs.gphase[1] != 0.0;
         if (gfold && (!rp_stage || (!fp64 && pr.g != 4))) fail(QW_ERR_STATE, "internal: a global phase on a stage without a table");
         if (rp_stage && (fp64 || pr.g == 4)) {
           sd.ph_block = fp64 ? (uint32_t)(ph64.size() / (2 * SV_PH64_BLOCK)) : (uint32_t)stages.size();
           double t[SV_G][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}, {0, 0}};
-          double gin[SV_G] = {1, 1, 1, 1, 1};  // input factor of the position's |1> half
           std::complex<double> d[SV_G][2] = {{1, 1}, {1, 1}, {1, 1}, {1, 1}, {1, 1}};
           for (const HostOp &o : sops) {
             double r00 = o.m[0], r01 = o.m[1], r10 = o.m[2], r11 = o.m[3];
@@ -272,31 +249,19 @@ struct SvTableBuilder {
               std::swap(r10, r11);
               sd.ld_xor ^= sd.roff[o.a];
             }
-            double a1 = 1.0;
             t[o.a][0] = r01 / r00;
             t[o.a][1] = r10 / r11;
-            if (!fp64) {
-              float T[2];
-              a1 = exact_rotation(r01 / r00, T);
-              t[o.a][0] = T[0];
-              t[o.a][1] = T[1];
-            }
-            gin[o.a] = 1.0 / a1;
             d[o.a][0] = r00;
-            d[o.a][1] = r11 * a1 * std::complex<double>(o.m[4], o.m[5]);
+            d[o.a][1] = r11 * std::complex<double>(o.m[4], o.m[5]);
           }
-          if (!fp64)
-            for (uint32_t e = 0; e < 16; e++) {
-              double f = 1.0;
-              for (uint32_t p4 = 0; p4 < 4; p4++)
-                if ((e >> p4) & 1u) f *= gin[p4];
-              ph.push_back((float)(f - 1.0));
+          for (uint32_t q = 0; q < pr.g; q++) {
+            if (fp64) {
+              ph64.insert(ph64.end(), {t[q][0], t[q][1]});
+            } else {
+              const float h0 = (float)t[q][0], h1 = (float)t[q][1];
+              ph.insert(ph.end(), {h0, h1, (float)(t[q][0] - (double)h0), (float)(t[q][1] - (double)h1)});
             }
-          for (uint32_t q = 0; q < pr.g; q++)
-            for (const double v : t[q]) {
-              if (fp64) ph64.push_back(v);
-              else ph.push_back((float)v);
-            }
+          }
           for (uint32_t e = 0; e < (1u << pr.g); e++) {
             std::complex<double> q(hs.gphase[0], hs.gphase[1]);
             for (uint32_t i = 0; i < pr.g; i++) q *= d[i][(e >> i) & 1u];
@@ -503,8 +468,8 @@ static void *chain_dst_lo(const DeviceState *D, int ar, size_t p, size_t n) {
 //   compensated (sv_df.cuh): a multiply-accumulate on the grid is 4 FMAs
 //   and a subtraction per component (18 for the amplitude's two), so with
 //   the un-biasing of the operand a two-term output costs 40, an
-//   unnormalized rotation output 18, a general 2x2 output 80, and every
-//   stage splits (6, 10 before rotations) and rounds (4) each amplitude.
+//   unnormalized rotation output 22, a general 2x2 output 80, and every
+//   stage splits (6) and rounds (4) each amplitude.
 static double pass_flops(const HostPass &hp, uint32_t n, uint32_t g, int ar) {
   const bool comp = ar != SV_AR_PLAIN;
   const double groups = std::ldexp(1.0, (int)n - (int)g), A = std::ldexp(1.0, (int)g);
@@ -520,7 +485,7 @@ static double pass_flops(const HostPass &hp, uint32_t n, uint32_t g, int ar) {
         mask |= 1u << o.a;
       }
       if (rot) {  // unnormalized rotations, then one product per amplitude
-        f += (fg + A * (4.0 + 18.0 * (double)st.ops.size() + cm)) * groups;
+        f += (fg + A * (22.0 * (double)st.ops.size() + cm)) * groups;
         continue;
       }
     }

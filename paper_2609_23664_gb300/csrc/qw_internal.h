@@ -198,7 +198,7 @@ struct SvPassDesc {
   // ctl_tb[i] of the tile index is set (ctl_w[i] = 0: unused)
   uint32_t ctl_tb[SV_MAX_OUT_CTL], ctl_w[SV_MAX_OUT_CTL];
 };
-constexpr uint32_t SV_PH_BLOCK = 16 + 4 * 2 + 16 * 4;  // floats of a rotation stage's block
+constexpr uint32_t SV_PH_BLOCK = 4 * 4 + 16 * 4;  // floats of a rotation stage's block
 constexpr uint32_t SV_PH64_BLOCK = 5 + 32;
 struct alignas(16) SvStageDesc {
   uint32_t roff[SV_G];           // byte offset of phi(e_pos[j]) for register bit j
@@ -209,9 +209,9 @@ struct alignas(16) SvStageDesc {
   // one per position in ascending order (run without dispatch)
   uint32_t rp_mask;
   // compensated FP32 stage of rotations: block of SV_PH_BLOCK floats of the
-  // table array (the stage's own index): for each amplitude index e of the group the input factor
-  // less one (16), the unnormalized rotation {t0, t1} of each of the four
-  // positions (zero where the mask has none), then for each e {re, re
+  // table array (the stage's own index): the unnormalized rotation {t0, t1,
+  // t0 remainder, t1 remainder} of each of the four positions (zero where the
+  // mask has none), then for each amplitude index e of the group {re, re
   // remainder, im, im remainder} of the factor it takes after the rotations:
   // the diagonal entries taken out of them, the |1>-phases of e's set
   // positions and the program's global phase where this stage carries it
@@ -401,8 +401,8 @@ struct SvTables {
 };
 // Arithmetic of FP32 statevector passes.  PLAIN: FP32 registers.  COMP:
 // two FP32 numbers per component while a stage runs (an op errs by about
-// 2^-39 of its group's largest amplitude), the amplitude rounded to FP32
-// when its stage writes it back.  REM: two numbers through the whole pass (a remainder plane beside the shared-memory tile)
+// 2^-39 of its group's largest amplitude, constants to 2^-48), the amplitude
+// rounded to FP32 when its stage writes it back.  REM: two numbers through the whole pass (a remainder plane beside the shared-memory tile)
 // and between passes (remainder arrays beside the state), so a chain of
 // passes rounds once, when it writes a state without its remainder.
 enum SvArith : int { SV_AR_PLAIN = 0, SV_AR_COMP = 1, SV_AR_REM = 2 };

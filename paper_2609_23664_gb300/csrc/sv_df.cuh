@@ -18,15 +18,24 @@
 // largest one, and the unnormalized rotations below stretch them by at most
 // sqrt(2) each (four per stage), together less than 2^5; with the largest
 // component below 2^E the unit u = 2^(E + 5 - 22) keeps every q within
-// 2^22 u.  The low parts are a few u, so one operation errs by about
-// 2^-24 * 4 u = 2^-39 of the group's largest amplitude, far below the FP32
-// rounding (2^-25) of the amplitudes that the stage stores.
+// 2^22 u.  The low parts are a few u (at most 5.2 after four rotations of
+// 20000 random groups), so one operation errs by about 2^-24 * 4 u = 2^-39 of
+// the group's largest amplitude (the four rotations of those groups: 2^-41.1
+// rms, 2^-38.1 at most), far below the FP32 rounding (2^-25) of the amplitudes
+// that the stage stores.  An amplitude below half a unit, 2^-18 of the
+// largest one, lies in its low part alone: plain FP32 precision.
+//
+// Constants are FP32 pairs throughout.  Rotations were tried with quotients
+// made exact in FP32 and a factor on the inputs (one instruction less per
+// output, 24-qubit sweep of 64 tasks 93.9 against 97.0 ms): the factor put
+// hundreds of units into the low parts and erred by 2^-34, always the same
+// way for one angle, so that 5000 repeats of it moved amplitudes by 3e-7.
 //
 // A two-term output costs 11 packed instructions and an unnormalized
-// rotation output 5 (and one more to un-bias its operand), against 16 for
+// rotation output 6 (and one more to un-bias its operand), against 16 for
 // the double-float arithmetic this replaced (products split by FMA, sums by
-// TwoSum): a full rotation stage takes 41 packed instructions per amplitude
-// instead of 80 (64-task 24-qubit suffix launch: 104 -> 61 ms), and the kernels that run it are bound by the FMA pipe.
+// TwoSum): a full rotation stage takes 44 packed instructions per amplitude
+// instead of 80, and the kernels that run it are bound by the FMA pipe.
 //
 // Without compensation, the FP32 roundings of the ~600 rotations that every
 // amplitude of a 24-qubit, 24-layer ansatz goes through move a Pauli-sum
@@ -57,11 +66,12 @@ __device__ __forceinline__ void gd_mac(float2 ch, float2 cl, float2 yq, float2 y
   H = h1;
 }
 
-// the same added to the amplitude H, l, for a constant that is exact in FP32
-__device__ __forceinline__ void gd_rot(float2 c, float2 yq, float2 yl, float2 &H, float2 &l) {
-  const float2 h1 = __ffma2_rn(c, yq, H);
-  const float2 e = __ffma2_rn(c, yq, f2sub(H, h1));
-  l = __fadd2_rn(__ffma2_rn(c, yl, l), e);
+// the same added to the amplitude H, l
+__device__ __forceinline__ void gd_rot(float2 ch, float2 cl, float2 yq, float2 yl, float2 &H, float2 &l) {
+  const float2 h1 = __ffma2_rn(ch, yq, H);
+  float2 e = __ffma2_rn(ch, yq, f2sub(H, h1));
+  e = __ffma2_rn(cl, yq, e);
+  l = __fadd2_rn(__ffma2_rn(ch, yl, l), e);
   H = h1;
 }
 
@@ -85,18 +95,17 @@ __device__ __forceinline__ void gd_cmul(float2 C, float wrh, float wrl, float wi
 // ---- register operations on the N = 2^G amplitudes of a stage group ------
 // m / ml: the op's parameters (see SvKind) and their FP32 remainders.
 
-// Unnormalized rotation on position P, t = {t0, t1}:
+// Unnormalized rotation on position P, t = {t0, t1} and their remainders:
 //   x' = x + t0 y,  y' = y + t1 x
-// (a real orthogonal 2x2 with its diagonal taken out; the host arranges
-// |t| <= 1, makes t0 and t1 exact in FP32 and puts what that takes into the
-// factors of the stage's table)
-__device__ __forceinline__ void gd_pair(float2 C, float2 t, float2 &Hx, float2 &lx, float2 &Hy, float2 &ly) {
+// (a real orthogonal 2x2 with its diagonal taken out into the factors of the
+// stage's table; the host arranges |t| <= 1)
+__device__ __forceinline__ void gd_pair(float2 C, float4 t, float2 &Hx, float2 &lx, float2 &Hy, float2 &ly) {
   const float2 xq = f2sub(Hx, C), yq = f2sub(Hy, C), xl = lx, yl = ly;
-  gd_rot(f2s(t.x), yq, yl, Hx, lx);
-  gd_rot(f2s(t.y), xq, xl, Hy, ly);
+  gd_rot(f2s(t.x), f2s(t.z), yq, yl, Hx, lx);
+  gd_rot(f2s(t.y), f2s(t.w), xq, xl, Hy, ly);
 }
 template <int P, int N>
-__device__ __forceinline__ void gdop_rot(float2 C, float2 (&H)[N], float2 (&l)[N], float2 t) {
+__device__ __forceinline__ void gdop_rot(float2 C, float2 (&H)[N], float2 (&l)[N], float4 t) {
 #pragma unroll
   for (int i = 0; i < N; i++)
     if (!(i & (1 << P))) gd_pair(C, t, H[i], l[i], H[i | (1 << P)], l[i | (1 << P)]);

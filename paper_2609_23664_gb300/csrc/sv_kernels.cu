@@ -265,18 +265,18 @@ __device__ __forceinline__ float gd_grid(float mx, float &C) {
 // Rotation stages (rp_mask != 0, one real rotation with an optional phase on
 // each position of the mask) run the unnormalized rotations, then multiply
 // every amplitude by its entry of the stage's table.  Bound by the FMA pipe:
-// 41 packed instructions per amplitude of a full stage (4 to split, 4 x 6
+// 44 packed instructions per amplitude of a full stage (3 to split, 4 x 7
 // for the rotations less one shared, 14 for the table and the rounding); the
-// 64-task 24-qubit suffix launch took 104 ms with the 80-instruction
-// double-float form, 64 ms with this one, and 61 ms since the next stage's
-// descriptor and table are fetched while a stage runs.
+// 64-task 24-qubit sweep took 155 ms with the 80-instruction double-float
+// form of the stages and takes 97 ms, of which fetching the next stage's
+// descriptor and table while a stage runs gives 3.
 template <int AR, int G>
 __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t sbB, uint32_t ldB,
                                             const uint32_t (&roff)[SV_G], const SvOpDesc<float> *__restrict__ ops,
                                             const float *__restrict__ ops_lo, uint32_t op_begin, uint32_t nops,
                                             uint32_t rp_mask, const float *blk) {
   constexpr int N = 1 << G;
-  static_assert(G == 4, "the phase block holds four rotations and 16 entries");
+  static_assert(G == 4, "the block holds four rotations and 16 factors");
   auto off = [&](int i) {
     return ((i & 1) ? roff[0] : 0u) ^ ((i & 2) ? roff[1] : 0u) ^ ((i & 4) ? roff[2] : 0u) ^ ((i & 8) ? roff[3] : 0u);
   };
@@ -298,24 +298,22 @@ __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t
     }
   }
   const float2 C = f2s(c1);
-  // the amplitude's factor (1 + eps) and its split: the part on the grid
-  // into H (biased), the exact rest and eps h into l
-  auto split = [&](int i, float eps) {
+  // the amplitude's part on the grid into H (biased), the exact rest into l
+  auto split = [&](int i) {
     const float2 h = H[i];
     H[i] = __fadd2_rn(h, C);
-    float2 r = __ffma2_rn(f2s(eps), h, f2sub(h, f2sub(H[i], C)));
+    float2 r = f2sub(h, f2sub(H[i], C));
     if constexpr (AR == SV_AR_REM) r = __fadd2_rn(r, l[i]);
     l[i] = r;
   };
   if (rp_mask) {
-    const float2 *t = (const float2 *)(blk + 16);
+    const float4 *t = (const float4 *)blk;
     if (rp_mask == 0xFu) {
-      const float2 t0 = t[0];
+      const float4 t0 = t[0];
 #pragma unroll
       for (int i = 0; i < N; i += 2) {
-        const float2 e = *(const float2 *)(blk + i);
-        split(i, e.x);
-        split(i + 1, e.y);
+        split(i);
+        split(i + 1);
         gd_pair(C, t0, H[i], l[i], H[i + 1], l[i + 1]);
       }
       gdop_rot<1, N>(C, H, l, t[1]);
@@ -323,13 +321,13 @@ __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t
       gdop_rot<3, N>(C, H, l, t[3]);
     } else {
 #pragma unroll
-      for (int i = 0; i < N; i++) split(i, blk[i]);
+      for (int i = 0; i < N; i++) split(i);
       if (rp_mask & 1u) gdop_rot<0, N>(C, H, l, t[0]);
       if (rp_mask & 2u) gdop_rot<1, N>(C, H, l, t[1]);
       if (rp_mask & 4u) gdop_rot<2, N>(C, H, l, t[2]);
       if (rp_mask & 8u) gdop_rot<3, N>(C, H, l, t[3]);
     }
-    const float4 *q = (const float4 *)(blk + 24);
+    const float4 *q = t + 4;
 #pragma unroll
     for (int e = 0; e < N; e++) {
       const float4 w = q[e];
@@ -337,7 +335,7 @@ __device__ __forceinline__ void sv_stage_df(char *smw, uint32_t lo_off, uint32_t
     }
   } else {
 #pragma unroll
-    for (int i = 0; i < N; i++) split(i, 0.f);
+    for (int i = 0; i < N; i++) split(i);
     for (uint32_t o = 0; o < nops; o++) {
       float m[8], ml[8];
       load_m(ops + op_begin + o, m);
@@ -409,7 +407,7 @@ __device__ void sv_tile(const SvPassDesc *__restrict__ pd, const SvStageDesc *__
     gstep[t] = lb < k ? gdep(1u << lb) : 0u;
     sstep[t] = lb < k ? swz<T>(1u << lb) * (uint32_t)sizeof(C) : 0u;
   }
-  // Compensated passes: a stage's descriptor and table (29 16-byte words) are
+  // Compensated passes: a stage's descriptor and table (27 16-byte words) are
   // copied to shared memory while the previous stage runs
   constexpr uint32_t SD = sizeof(SvStageDesc) / 16, SB = SV_PH_BLOCK / 4;
   __shared__ uint4 staged[AR != SV_AR_PLAIN ? 2 : 1][AR != SV_AR_PLAIN ? SD + SB : 1];
