@@ -54,7 +54,7 @@ template <typename T> struct AccOf;
 template <> struct AccOf<float> { typedef DFAcc t; };
 template <> struct AccOf<double> { typedef DAcc t; };
 
-// Warp sums of the lanes' accumulators and of their norms.  FP32 blocks add
+// Warp sums of the lanes' accumulators.  FP32 blocks add
 // in double-float: FP64 adds run at 1/64 of the FP32 rate, and a block is
 // short enough (13 groups per class) that 12 of them per thread showed.
 __device__ __forceinline__ double en_warp_total(DFAcc a) {
@@ -68,12 +68,6 @@ __device__ __forceinline__ double en_warp_total(DFAcc a) {
 }
 __device__ __forceinline__ double en_warp_sum(double v);
 __device__ __forceinline__ double en_warp_total(DAcc a) { return en_warp_sum(a.v); }
-__device__ __forceinline__ double en_warp_total_norm(float v) {
-  DFAcc a;
-  a.hi = v;
-  return en_warp_total(a);
-}
-__device__ __forceinline__ double en_warp_total_norm(double v) { return en_warp_sum(v); }
 
 __device__ __forceinline__ double en_warp_sum(double v) {
 #pragma unroll
@@ -165,6 +159,26 @@ __device__ __forceinline__ double en_pairs(const double2 (&a)[16], uint32_t zz) 
     s1 = fma(IM ? -py : py, IM ? a[i].x : a[i].y, s1);
   }
   return s0 + s1;
+}
+// Squared norm of the amplitudes [LO, LO + CNT), added in a tree: the error of
+// 32 FP32 squares added one after another is the same in every thread of a
+// state of constant amplitude (5e-7 of the norm, and of every energy).
+template <int LO, int CNT, int N>
+__device__ __forceinline__ float2 en_squares(const float2 (&a)[N]) {
+  if constexpr (CNT == 2) return __ffma2_rn(a[LO], a[LO], __fmul2_rn(a[LO + 1], a[LO + 1]));
+  else return __fadd2_rn(en_squares<LO, CNT / 2>(a), en_squares<LO + CNT / 2, CNT / 2>(a));
+}
+template <int N>
+__device__ __forceinline__ float en_norm(const float2 (&a)[N]) {
+  const float2 s = en_squares<0, N>(a);
+  return s.x + s.y;
+}
+template <int N>
+__device__ __forceinline__ double en_norm(const double2 (&a)[N]) {
+  double s = 0;
+#pragma unroll
+  for (int k = 0; k < N; k++) s += a[k].x * a[k].x + a[k].y * a[k].y;
+  return s;
 }
 // the term's sign data in the form its precision takes
 template <typename T> struct EnSign;
@@ -263,8 +277,7 @@ __device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const 
   while (c + 1 < ce && tab.classes[c + 1].block_begin <= jb) c++;
   const EnClass K = tab.classes[c];
   const C *psi = (const C *)J.state;
-  typename AccOf<T>::t acc;
-  T nrm = 0;
+  typename AccOf<T>::t acc, nrm;
   const uint32_t n_rep = 1u << (J.n - EN_RANK - (PAIR ? 1 : 0));
 #pragma unroll 1
   for (uint32_t it = 0; it < (1u << J.iter_bits); it++) {
@@ -295,12 +308,7 @@ __device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const 
           a[i] = en_ld<NC>(psi + x);
         }
       }
-      if (w.w & EN_GROUP_NORM) {
-        T s = 0;
-#pragma unroll
-        for (int k = 0; k < N; k++) s += a[k].x * a[k].x + a[k].y * a[k].y;
-        nrm += s;
-      }
+      if (w.w & EN_GROUP_NORM) nrm.add(en_norm(a));
       uint32_t t = w.y;
       // the first terms flip the basis masks, one each: straight-line code, a
       // uniform branch or two each (random Hamiltonians hold few others)
@@ -322,7 +330,7 @@ __device__ __forceinline__ void energy_block(const EnJob &J, uint32_t jb, const 
     }
   }
   __shared__ double en_red[2][8];
-  const double e = en_warp_total(acc), nn = en_warp_total_norm(nrm);
+  const double e = en_warp_total(acc), nn = en_warp_total(nrm);
   const int w = threadIdx.x >> 5, ln = threadIdx.x & 31;
   if (ln == 0) { en_red[0][w] = e; en_red[1][w] = nn; }
   __syncthreads();
