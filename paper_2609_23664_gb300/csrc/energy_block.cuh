@@ -54,26 +54,29 @@ template <typename T> struct AccOf;
 template <> struct AccOf<float> { typedef DFAcc t; };
 template <> struct AccOf<double> { typedef DAcc t; };
 
-// Warp sums of the lanes' accumulators.  FP32 blocks add
-// in double-float: FP64 adds run at 1/64 of the FP32 rate, and a block is
-// short enough (13 groups per class) that 12 of them per thread showed.
-__device__ __forceinline__ double en_warp_total(DFAcc a) {
+__device__ __forceinline__ double en_warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+// Warp sums of the lanes' accumulators.  FP32 blocks add in double-float:
+// FP64 adds run at 1/64 of the FP32 rate, and a block is short enough (13
+// groups per class) that 12 of them per thread showed.  Where 32 lanes'
+// sums leave the FP32 range (amplitudes of about 10^18) they add in FP64.
+__device__ __forceinline__ double en_warp_total(const DFAcc in) {
+  DFAcc a = in;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
     a.add(h);
     a.lo += l;
   }
+  if (__any_sync(0xffffffffu, !(fabsf(a.hi) <= 3.402823466e38f)))
+    // (an infinite sum has no low part)
+    return en_warp_sum(fabsf(in.hi) <= 3.402823466e38f ? in.value() : (double)in.hi);
   return a.value();
 }
-__device__ __forceinline__ double en_warp_sum(double v);
 __device__ __forceinline__ double en_warp_total(DAcc a) { return en_warp_sum(a.v); }
-
-__device__ __forceinline__ double en_warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
 
 // NC: the state is read-only for the whole launch (read-only cache path);
 // otherwise it was written earlier in the same launch by other CTAs and is
