@@ -421,7 +421,10 @@ smp_blocksum_kernel(const SmpSource *__restrict__ srcs, uint32_t n_src, uint32_t
 // one CTA per source: boff[b] = sum of the blocks before b, the entry after
 // the last block is the total.  Each thread adds a run of blocks in order,
 // the runs' sums are scanned across the CTA.  (One thread per source, block
-// by block, took 1.87 ms for the 16384 blocks of 26 qubits.)
+// by block, took 1.87 ms for the 16384 blocks of 26 qubits.)  The scan rounds
+// in another order than the runs do, so the offsets may step by an ulp from
+// one run to the next: an empty block takes the offset of the next block that
+// is not empty, so that no target falls into it.
 constexpr int SMP_OFF_THREADS = 256;
 __global__ void __launch_bounds__(SMP_OFF_THREADS)
 smp_offsets_kernel(const SmpSource *__restrict__ srcs, const double *__restrict__ bsum,
@@ -442,6 +445,8 @@ smp_offsets_kernel(const SmpSource *__restrict__ srcs, const double *__restrict_
   // exclusive scan of the runs' sums: within a warp, then of the warps
   __shared__ double wsum[SMP_OFF_THREADS / 32];
   __shared__ int64_t wlast[SMP_OFF_THREADS / 32];
+  __shared__ unsigned wfilled[SMP_OFF_THREADS / 32];
+  __shared__ double base[SMP_OFF_THREADS + 1];  // offset of each run, the total
   double incl = acc;
 #pragma unroll
   for (int d = 1; d < 32; d *= 2) {
@@ -450,21 +455,36 @@ smp_offsets_kernel(const SmpSource *__restrict__ srcs, const double *__restrict_
   }
   double excl = __shfl_up_sync(0xffffffffu, incl, 1);
   if ((t & 31) == 0) excl = 0;
+  const uint32_t end = last >= 0 ? (uint32_t)(last >> SMP_BLOCK_BITS) + 1 : b0;  // past the run's last filled block
+  const unsigned filled = __ballot_sync(0xffffffffu, last >= 0);
 #pragma unroll
   for (int d = 16; d > 0; d >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, d));
   if ((t & 31) == 31) wsum[t >> 5] = incl;
-  if ((t & 31) == 0) wlast[t >> 5] = last;
+  if ((t & 31) == 0) {
+    wlast[t >> 5] = last;
+    wfilled[t >> 5] = filled;
+  }
   __syncthreads();
   double before = 0;
   for (uint32_t w = 0; w < (t >> 5); w++) before = before + wsum[w];
   acc = before + excl;
+  base[t] = acc;
+  if (t == SMP_OFF_THREADS - 1) base[SMP_OFF_THREADS] = before + incl;
+  __syncthreads();
 #pragma unroll 8
-  for (uint32_t b = b0; b < b1; b++) {
+  for (uint32_t b = b0; b < end; b++) {
     o[b] = acc;
     acc = acc + bsum[S.block_begin + b];
   }
+  if (end < b1) {  // the run ends with empty blocks: the next filled run's offset
+    uint32_t w = t >> 5;
+    unsigned m = (t & 31) == 31 ? 0u : wfilled[w] >> ((t & 31) + 1) << ((t & 31) + 1);
+    while (!m && ++w < SMP_OFF_THREADS / 32) m = wfilled[w];
+    const double next = base[m ? 32 * w + (uint32_t)__ffs(m) - 1 : SMP_OFF_THREADS];
+    for (uint32_t b = end; b < b1; b++) o[b] = next;
+  }
   if (t == SMP_OFF_THREADS - 1) {
-    o[S.n_blocks] = before + incl;
+    o[S.n_blocks] = base[SMP_OFF_THREADS];
     for (int w = 0; w < SMP_OFF_THREADS / 32; w++) last = max(last, wlast[w]);
     lastnz[s] = last;
   }

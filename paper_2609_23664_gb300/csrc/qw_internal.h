@@ -467,7 +467,7 @@ void launch_energy(bool fp64, bool pair, const EnTables &t, uint32_t n_jobs, uin
                    void *stream);
 // the reduction alone, for partials written by the persistent launch
 void launch_energy_reduce(const EnJob *jobs, uint32_t n_jobs, const double *partials, void *stream);
-// sampling: block sums -> per-source sequential offsets -> shots
+// sampling: block sums -> offsets by a scan per source -> shots
 void launch_sampling(bool fp64, const SmpSource *srcs, uint32_t n_src, uint32_t total_blocks,
                      double *bsum, int32_t *blast, double *boff, int64_t *lastnz,
                      const SmpShot *shots, uint32_t n_shots, void *stream);
