@@ -30,3 +30,10 @@ def test_ctas_fit_the_workspace(batch):
     have = scratch(batch)
     for b in range(max(1, batch - 4000), batch + 1):
         assert ctas(b) * N_PARTIAL <= have, b
+
+
+@pytest.mark.parametrize("batch", [1, 31, 100, 3199, 3200, 3201, 6400, 65536, 65537, 1 << 24, (1 << 32) - 1])
+def test_no_cta_takes_more_than_32_samples(batch):
+    # samples of a CTA run one after another, in gradients and in forward passes
+    ctas = _fn("_ZN2qw13mlp_grad_ctasEj", ctypes.c_uint32)(batch)
+    assert batch <= 32 * ctas and ctas <= batch
