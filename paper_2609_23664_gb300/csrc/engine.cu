@@ -58,6 +58,14 @@ void launch_copy(const void *src, void *dst, size_t bytes, void *stream) {
 // ---------------------------------------------------------------------------
 // device-side tables of a set of statevector programs
 // ---------------------------------------------------------------------------
+// A stage of one rotation without a phase runs as a general op: its two-term
+// outputs (compensated: 17 packed instructions per amplitude with the split
+// and the rounding, FP64: 4 operations) cost less than an unnormalized
+// rotation and the factors of the table (24 and 6).
+static bool lone_rotation(const HostStage &st) {
+  return st.ops.size() == 1 && st.ops[0].kind == K_R && st.gphase[0] == 1.0 && st.gphase[1] == 0.0;
+}
+
 struct SvTableBuilder {
   std::vector<SvPassDesc> passes;
   std::vector<SvStageDesc> stages;
@@ -214,6 +222,7 @@ struct SvTableBuilder {
           if ((o.kind != K_RP && o.kind != K_R) || (rp_mask & (1u << o.a))) { rp_stage = false; break; }
           rp_mask |= 1u << o.a;
         }
+        if ((fp64 || pr.g == 4) && lone_rotation(hs)) rp_stage = false;
         if (rp_stage) {
           std::sort(sops.begin(), sops.end(), [](const HostOp &x, const HostOp &y) { return x.a < y.a; });
           for (HostOp &o : sops)
@@ -484,7 +493,7 @@ static double pass_flops(const HostPass &hp, uint32_t n, uint32_t g, int ar) {
         rot = rot && (o.kind == K_RP || o.kind == K_R) && !(mask & (1u << o.a));
         mask |= 1u << o.a;
       }
-      if (rot) {  // unnormalized rotations, then one product per amplitude
+      if (rot && !lone_rotation(st)) {  // unnormalized rotations, then one product per amplitude
         f += (fg + A * (22.0 * (double)st.ops.size() + cm)) * groups;
         continue;
       }
