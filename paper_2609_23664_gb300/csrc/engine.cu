@@ -2182,13 +2182,15 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   cudaStream_t s = (cudaStream_t)stream;
   const bool fp64 = mode == QW_MODE_SV_FP64;
   // FP32: compensated arithmetic with the remainder kept between passes, so
-  // the state is rounded once, by the last pass
-  const int ar = fp64 ? SV_AR_PLAIN : SV_AR_REM;
+  // the state is rounded once, by the last pass (none where nothing rounds)
+  int ar = fp64 ? SV_AR_PLAIN : SV_AR_REM;
   uint64_t n2 = 0;
   for (uint64_t i = 0; i < n_gates; i++) n2 += is_two_qubit_op(gates[i].op) ? 1 : 0;
   TileConfig tc = E->tile_config(n, fp64, SV_AR_COMP, gate_mix(n2, n_gates));
-  tc.k_max = std::min<uint32_t>(tc.k_max, sv_max_tile(ar, fp64));
+  tc.k_max = sv_permutes(gates, n_gates) ? (uint32_t)sv_max_tile(SV_AR_COMP, fp64)
+                                         : std::min<uint32_t>(tc.k_max, sv_max_tile(ar, fp64));
   SvProgram pr = fuse_sv(gates, n_gates, n, tc, fp64);
+  if (ar == SV_AR_REM && sv_exact(pr)) ar = SV_AR_COMP;
   if (pr.passes.empty()) {
     if (!init) return QW_OK;
     HostPass hp;

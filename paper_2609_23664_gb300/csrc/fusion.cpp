@@ -449,6 +449,23 @@ SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const 
   return prog;
 }
 
+bool sv_permutes(const qw_gate *gates, uint64_t n_gates) {
+  for (uint64_t i = 0; i < n_gates; i++)
+    if (gates[i].op != QW_OP_X && gates[i].op != QW_OP_CNOT && gates[i].op != QW_OP_SWAP) return false;
+  return true;
+}
+bool sv_exact(const SvProgram &p) {
+  auto unit = [](double v) { return v == 0.0 || v == 1.0 || v == -1.0; };
+  for (const HostPass &ps : p.passes)
+    for (const HostStage &st : ps.stages) {
+      if (!unit(st.gphase[0]) || !unit(st.gphase[1])) return false;
+      for (const HostOp &o : st.ops)
+        for (double v : o.m)
+          if (!unit(v)) return false;
+    }
+  return true;
+}
+
 uint32_t estimate_passes(uint64_t n_gates, uint32_t n, const TileConfig &tc, double gates_per_pass) {
   if (n_gates == 0) return 0;
   if (n <= tc.k_max) return 1;

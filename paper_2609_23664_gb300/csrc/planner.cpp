@@ -1046,9 +1046,12 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
     } else {
       T.copy_gates(tp.begin, T.n_gates, buf);
       TileConfig tc = C.tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
+      if (!P->opts.tile_qubits && sv_permutes(buf.data(), buf.size()))
+        tc.k_max = sv_max_tile(T.mode == QW_MODE_SV_FP64 ? SV_AR_PLAIN : plan_ar_batch(P), T.mode == QW_MODE_SV_FP64);
       tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc, T.mode == QW_MODE_SV_FP64);
+      const bool exact = sv_exact(tp.sv);
       tp.chain = T.mode == QW_MODE_SV_FP32 && plan_ar_batch(P) == SV_AR_COMP &&
-                 (!P->opts.batched || tp.sv.passes.size() > (size_t)SV_COMP_MAX_BATCH_PASSES);
+                 (!P->opts.batched || (!exact && tp.sv.passes.size() > (size_t)SV_COMP_MAX_BATCH_PASSES));
       if (tp.chain) {
         tc = C.tiles(tp.n_eff, false, true);
         tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc);

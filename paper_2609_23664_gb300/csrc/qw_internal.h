@@ -236,6 +236,14 @@ static_assert(sizeof(SvOpDesc<float>) == 48 && sizeof(SvOpDesc<double>) == 80, "
 // Fusion planner: gates -> passes -> stages (host).
 // (fp64: for FP64 passes, whose first rotation stage can carry the global phase)
 SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const TileConfig &tc, bool fp64 = false);
+// Whether gates only permute amplitudes.  Such programs have no stages, so
+// they take the widest tiles instead of those chosen for rotations (60 CNOTs,
+// 24 FP32 qubits: 590 -> 259 us with the remainder left out too, 12 FP64
+// qubits: 33 -> 12 us).
+bool sv_permutes(const qw_gate *gates, uint64_t n_gates);
+// Whether a program only permutes amplitudes and multiplies them by +-1 and
+// +-i: its passes round nothing, so they need no remainder.
+bool sv_exact(const SvProgram &p);
 // Number of passes a segment would take (cheap estimate used by the planner).
 uint32_t estimate_passes(uint64_t n_gates, uint32_t n, const TileConfig &tc, double gates_per_pass);
 // Gate matrix in double precision (host). Returns false for non-1q ops.
