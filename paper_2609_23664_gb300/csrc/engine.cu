@@ -357,6 +357,7 @@ struct Wave {
   std::vector<uint32_t> tasks;            // tasks run in this wave (own buffers)
   std::vector<uint32_t> obs_tasks;        // tasks whose observables are evaluated in this wave
   std::vector<SvJob> jobs;                // pass jobs, in list order
+  bool few = false;                       // at most SV_FEW_TILES tiles side by side
   bool fused_energy = false;              // energy blocks run inside the persistent launch
   uint32_t seg_bits = 0;
   std::vector<SvSeg> segs;
@@ -398,6 +399,7 @@ struct DeviceState {
     bool fp64 = false;
     int ar = SV_AR_PLAIN;
     uint32_t k_max = 5, seg_bits = 0, total_items = 0;
+    bool few = false;  // at most SV_FEW_TILES tiles side by side
     int grid = 0;
     size_t n_jobs = 0, ctr_words = 0;
     SvJob *d_jobs = nullptr;
@@ -792,7 +794,11 @@ static void prepare(qw_plan *P) {
         B.fp64 = prec == QW_MODE_SV_FP64;
         B.k_max = kmax;
         B.ar = ar;
-        B.grid = sv_batch_grid(B.fp64, kmax, E->sm_count, ar);
+        std::vector<uint64_t> tiles(max_level + 1, 0);  // of the siblings of each level
+        for (size_t m = 0; m < P->mats.size(); m++)
+          if (P->mats[m].mode == prec) tiles[level[m]] += 1ull << (P->mats[m].n_eff - std::min(P->mats[m].n_eff, kmax));
+        B.few = *std::max_element(tiles.begin(), tiles.end()) <= SV_FEW_TILES;
+        B.grid = sv_batch_grid(B.fp64, kmax, E->sm_count, ar, false, B.few);
         B.seg_bits = segment_bits(jobs);
         std::vector<SvSeg> segs;
         build_segments(jobs, jobs.size(), B.seg_bits, 2ull * (uint64_t)B.grid, segs);
@@ -1100,7 +1106,8 @@ static void prepare(qw_plan *P) {
       std::vector<SvJob> up = W.jobs;
       W.fused_energy =
           !W.per_pass && W.ar != SV_AR_REM && P->opts.fuse_energy && !W.en.empty() && sv_threads_for_k(W.k_max, W.ar, fp64) == 128;
-      W.grid = !W.per_pass ? sv_batch_grid(fp64, W.k_max, E->sm_count, W.ar, W.fused_energy) : 0;
+      W.few = ((uint64_t)W.tasks.size() << (n_eff - std::min(n_eff, W.k_max))) <= SV_FEW_TILES;
+      W.grid = !W.per_pass ? sv_batch_grid(fp64, W.k_max, E->sm_count, W.ar, W.fused_energy, W.few) : 0;
       if (W.fused_energy) {
         std::vector<SvJob> ej;
         for (size_t e = 0; e < W.en.size(); e++) {
@@ -1385,7 +1392,7 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
     for (const DeviceState::MatBatch &B : D->mat_batches) {
       CK(cudaMemsetAsync(B.d_ctr, 0, B.ctr_words * sizeof(unsigned int), s));
       launch_sv_batch(B.fp64, B.fp64 ? D->t64 : D->t32, B.d_jobs, B.d_segs, B.seg_bits, B.total_items, B.k_max,
-                      B.d_ctr, EnTables{}, B.grid, s, B.ar);
+                      B.d_ctr, EnTables{}, B.grid, s, B.ar, B.few);
       nl += 1;
     }
     // each boundary rounded once into the other precision its consumers use
@@ -1420,7 +1427,7 @@ static void enqueue(qw_plan *P, cudaStream_t s, bool capturing) {
         const EnTables et =
             W.fused_energy ? EnTables{W.d_en, D->d_classes, D->d_groups, D->d_terms, D->d_partials} : EnTables{};
         launch_sv_batch(W.fp64, T, W.d_jobs, W.d_segs, W.seg_bits, W.total_items, W.k_max, W.d_ctr, et,
-                        W.grid, s, W.ar);
+                        W.grid, s, W.ar, W.few);
         nl += 1;
       }
     } else {
@@ -2187,7 +2194,7 @@ qw_status sv_apply_dev(Engine *E, uint32_t mode, uint32_t n, void *state, const 
   uint64_t n2 = 0;
   for (uint64_t i = 0; i < n_gates; i++) n2 += is_two_qubit_op(gates[i].op) ? 1 : 0;
   TileConfig tc = E->tile_config(n, fp64, SV_AR_COMP, gate_mix(n2, n_gates));
-  tc.k_max = sv_permutes(gates, n_gates) ? (uint32_t)sv_max_tile(SV_AR_COMP, fp64)
+  tc.k_max = sv_permutes(gates, n_gates) ? sv_permute_tile(n, fp64, tc.k_max)
                                          : std::min<uint32_t>(tc.k_max, sv_max_tile(ar, fp64));
   SvProgram pr = fuse_sv(gates, n_gates, n, tc, fp64);
   if (ar == SV_AR_REM && sv_exact(pr)) ar = SV_AR_COMP;

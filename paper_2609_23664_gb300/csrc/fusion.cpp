@@ -454,6 +454,10 @@ bool sv_permutes(const qw_gate *gates, uint64_t n_gates) {
     if (gates[i].op != QW_OP_X && gates[i].op != QW_OP_CNOT && gates[i].op != QW_OP_SWAP) return false;
   return true;
 }
+uint32_t sv_permute_tile(uint32_t n, bool fp64, uint32_t tuned) {
+  const uint32_t wide = (uint32_t)sv_max_tile(SV_AR_COMP, fp64);
+  return fp64 && n > wide ? std::max(tuned, 12u) : std::max(tuned, wide);
+}
 bool sv_exact(const SvProgram &p) {
   auto unit = [](double v) { return v == 0.0 || v == 1.0 || v == -1.0; };
   for (const HostPass &ps : p.passes)

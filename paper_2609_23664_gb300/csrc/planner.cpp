@@ -1047,7 +1047,7 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
       T.copy_gates(tp.begin, T.n_gates, buf);
       TileConfig tc = C.tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
       if (!P->opts.tile_qubits && sv_permutes(buf.data(), buf.size()))
-        tc.k_max = sv_max_tile(T.mode == QW_MODE_SV_FP64 ? SV_AR_PLAIN : plan_ar_batch(P), T.mode == QW_MODE_SV_FP64);
+        tc.k_max = sv_permute_tile(tp.n_eff, T.mode == QW_MODE_SV_FP64, tc.k_max);
       tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc, T.mode == QW_MODE_SV_FP64);
       const bool exact = sv_exact(tp.sv);
       tp.chain = T.mode == QW_MODE_SV_FP32 && plan_ar_batch(P) == SV_AR_COMP &&

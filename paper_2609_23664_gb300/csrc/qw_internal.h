@@ -240,7 +240,10 @@ SvProgram fuse_sv(const qw_gate *gates, uint64_t n_gates, uint32_t n_eff, const 
 // they take the widest tiles instead of those chosen for rotations (60 CNOTs,
 // 24 FP32 qubits: 590 -> 259 us with the remainder left out too, 12 FP64
 // qubits: 33 -> 12 us).
+// (FP64 ones keep 12 qubits above 13: a wider tile leaves one CTA per SM, one
+// CNOT at 24 qubits 97 us against 91.)
 bool sv_permutes(const qw_gate *gates, uint64_t n_gates);
+uint32_t sv_permute_tile(uint32_t n, bool fp64, uint32_t tuned);
 // Whether a program only permutes amplitudes and multiplies them by +-1 and
 // +-i: its passes round nothing, so they need no remainder.
 bool sv_exact(const SvProgram &p);
@@ -450,7 +453,9 @@ struct SvSeg {
 // kernel attributes (dynamic shared memory limits); the first failure is returned
 cudaError_t sv_init_attrs();
 cudaError_t tab_init_attrs();
-int sv_threads_for_k(uint32_t k, int ar = SV_AR_PLAIN, bool fp64 = false);
+// few: the launch's independent tiles number at most SV_FEW_TILES
+constexpr uint32_t SV_FEW_TILES = 128;
+int sv_threads_for_k(uint32_t k, int ar = SV_AR_PLAIN, bool fp64 = false, bool few = false);
 size_t sv_smem_bytes(bool fp64, uint32_t k, int ar = SV_AR_PLAIN);
 // one pass over one state (grid = tiles); ar applies to FP32 states; the
 // remainder arrays (float2 per amplitude, NULL allowed) to SV_AR_REM only
@@ -464,8 +469,8 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
 // en.jobs: non-NULL when the list holds energy jobs.
 void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSeg *segs, uint32_t seg_bits,
                      uint32_t total_items, uint32_t k_max, unsigned int *counters, const EnTables &en,
-                     int grid, void *stream, int ar = SV_AR_PLAIN);
-int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar = SV_AR_PLAIN, bool energy = false);
+                     int grid, void *stream, int ar = SV_AR_PLAIN, bool few = false);
+int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar = SV_AR_PLAIN, bool energy = false, bool few = false);
 void launch_copy(const void *src, void *dst, size_t bytes, void *stream);
 
 // energy: per-block partials (2 doubles per block), then one reduction

@@ -744,12 +744,16 @@ sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restr
 // (FP32) or five (FP64) positions.  Threads: every thread owns at least two
 // stage groups of a 2^13 tile (128 threads; 256 for plain FP32 passes with
 // four-position stages, whose register budget fits three such CTAs per
-// SM).
+// SM).  Passes with a remainder whose tiles leave SMs idle anyway (`few`) give
+// every stage group its own thread, on CTAs that have an SM to themselves: a
+// pass then lasts as long as one tile.  (Tiles come in powers of two, so at
+// most SV_FEW_TILES of them fit the 152 SMs at once.)
 constexpr int SV_NT_PLAIN32 = (SV_G_PLAIN32 == 4) ? 256 : 128;
-int sv_threads_for_k(uint32_t k, int ar, bool fp64) {
+int sv_threads_for_k(uint32_t k, int ar, bool fp64, bool few) {
   const uint32_t G = (uint32_t)sv_stage_width(ar, fp64);
-  const uint32_t g = 1u << (k - G - 1);
-  const uint32_t cap = (!fp64 && ar == SV_AR_PLAIN) ? (uint32_t)SV_NT_PLAIN32 : 128u;
+  const bool wide = few && !fp64 && ar == SV_AR_REM;
+  const uint32_t g = 1u << (wide ? k - G : k - G - 1);
+  const uint32_t cap = wide ? 256u : (!fp64 && ar == SV_AR_PLAIN) ? (uint32_t)SV_NT_PLAIN32 : 128u;
   return (int)(g < 32 ? 32 : (g > cap ? cap : g));
 }
 size_t sv_smem_bytes(bool fp64, uint32_t k, int ar) {
@@ -760,10 +764,11 @@ size_t sv_smem_bytes(bool fp64, uint32_t k, int ar) {
 // a 128-register build (four CTAs per SM) for tiles of at most 12 qubits
 typedef void (*SvBatchKernel)(SvTables, const SvJob *, const SvSeg *, uint32_t, uint32_t, unsigned int *, EnTables);
 template <bool EN>
-static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar) {
+static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar, bool few = false) {
   if (fp64) return sv_batch_kernel<double, 1, SV_AR_PLAIN, 128, EN>;
   if (ar == SV_AR_COMP) return sv_batch_kernel<float, 3, SV_AR_COMP, 128, EN>;
-  if (ar == SV_AR_REM) return sv_batch_kernel<float, 3, SV_AR_REM, 128, false>;
+  if (ar == SV_AR_REM)
+    return few ? sv_batch_kernel<float, 1, SV_AR_REM, 256, false> : sv_batch_kernel<float, 3, SV_AR_REM, 128, false>;
   if constexpr (SV_G_PLAIN32 == 4) return sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, false>;
   else
     return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, EN>
@@ -777,12 +782,14 @@ cudaError_t sv_init_attrs() {
   const void *k[] = {(const void *)sv_pass_kernel<float, SV_AR_PLAIN, SV_NT_PLAIN32, 3>,
                      (const void *)sv_pass_kernel<float, SV_AR_COMP, 128, 3>,
                      (const void *)sv_pass_kernel<float, SV_AR_REM, 128, 3>,
+                     (const void *)sv_pass_kernel<float, SV_AR_REM, 256, 1>,
                      (const void *)sv_pass_kernel<double, SV_AR_PLAIN, 128, 1>,
                      (const void *)batch_kernel_of<false>(false, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 12, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 13, SV_AR_COMP),
                      (const void *)batch_kernel_of<false>(true, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 12, SV_AR_REM),
+                     (const void *)batch_kernel_of<false>(false, 12, SV_AR_REM, true),
                      (const void *)batch_kernel_of<true>(false, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<true>(false, 12, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<true>(false, 13, SV_AR_COMP),
@@ -798,7 +805,8 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
                     void *dst, void *stream, int ar, const void *src_lo, void *dst_lo) {
   const uint32_t tiles = 1u << (n - k);
   if (fp64) ar = SV_AR_PLAIN;
-  const int threads = sv_threads_for_k(k, ar, fp64);
+  const bool few = tiles <= SV_FEW_TILES;
+  const int threads = sv_threads_for_k(k, ar, fp64, few);
   const size_t smem = sv_smem_bytes(fp64, k, ar);
   cudaStream_t s = (cudaStream_t)stream;
   const float2 *sl = (const float2 *)src_lo;
@@ -807,8 +815,8 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
     sv_pass_kernel<double, SV_AR_PLAIN, 128, 1><<<tiles, threads, smem, s>>>(t, pass_idx, (const double2 *)src,
                                                                               (double2 *)dst, nullptr, nullptr);
   } else if (ar == SV_AR_REM) {
-    sv_pass_kernel<float, SV_AR_REM, 128, 3><<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src,
-                                                                           (float2 *)dst, sl, dl);
+    (few ? sv_pass_kernel<float, SV_AR_REM, 256, 1> : sv_pass_kernel<float, SV_AR_REM, 128, 3>)
+        <<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src, (float2 *)dst, sl, dl);
   } else if (ar == SV_AR_COMP) {
     sv_pass_kernel<float, SV_AR_COMP, 128, 3><<<tiles, threads, smem, s>>>(t, pass_idx, (const float2 *)src,
                                                                             (float2 *)dst, nullptr, nullptr);
@@ -818,12 +826,12 @@ void launch_sv_pass(bool fp64, const SvTables &t, uint32_t pass_idx, uint32_t k,
   }
 }
 
-int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy) {
+int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy, bool few) {
   if (fp64) ar = SV_AR_PLAIN;
-  const int threads = sv_threads_for_k(k, ar, fp64);
+  const int threads = sv_threads_for_k(k, ar, fp64, few);
   const size_t smem = sv_smem_bytes(fp64, k, ar);
   int per_sm = 0;
-  const SvBatchKernel f = energy ? batch_kernel_of<true>(fp64, k, ar) : batch_kernel_of<false>(fp64, k, ar);
+  const SvBatchKernel f = energy ? batch_kernel_of<true>(fp64, k, ar) : batch_kernel_of<false>(fp64, k, ar, few);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, threads, smem);
   if (per_sm < 1) per_sm = 1;
   return per_sm * sm_count;
@@ -831,12 +839,12 @@ int sv_batch_grid(bool fp64, uint32_t k, int sm_count, int ar, bool energy) {
 
 void launch_sv_batch(bool fp64, const SvTables &t, const SvJob *jobs, const SvSeg *segs, uint32_t seg_bits,
                      uint32_t total_items, uint32_t k_max, unsigned int *counters, const EnTables &en,
-                     int grid, void *stream, int ar) {
+                     int grid, void *stream, int ar, bool few) {
   if (fp64) ar = SV_AR_PLAIN;
-  const int threads = sv_threads_for_k(k_max, ar, fp64);
+  const int threads = sv_threads_for_k(k_max, ar, fp64, few);
   const size_t smem = sv_smem_bytes(fp64, k_max, ar);
   const SvBatchKernel f =
-      en.jobs ? batch_kernel_of<true>(fp64, k_max, ar) : batch_kernel_of<false>(fp64, k_max, ar);
+      en.jobs ? batch_kernel_of<true>(fp64, k_max, ar) : batch_kernel_of<false>(fp64, k_max, ar, few);
   f<<<grid, threads, smem, (cudaStream_t)stream>>>(t, jobs, segs, seg_bits, total_items, counters, en);
 }
 
