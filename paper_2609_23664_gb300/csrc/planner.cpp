@@ -460,6 +460,29 @@ struct PlanCtx {
     return tc;
   }
 
+  // The tuner times a shape on as many states as keep the chip busy.  Few
+  // compensated states (at most SV_FEW_STATES_TILES tiles of 2^12 in all, two
+  // rounds of the resident CTAs) are bound by the length of a pass instead,
+  // which half the tile halves: random circuits of 100 gates at 18 qubits, one
+  // task 256 us in 2^13 tiles and 140 us in 2^12, 8 tasks 283 and 194; 24
+  // tasks of 60 gates 312 and 308, 8 tasks at 20 qubits 349 and 380.
+  std::map<uint32_t, uint64_t> states_of;  // compensated FP32 tasks by register size
+  bool few_states(uint32_t n_eff) {
+    if (states_of.empty())
+      for (const TaskData &T : W.tasks)
+        if (T.mode == QW_MODE_SV_FP32) states_of[std::max<uint32_t>(T.n, SV_G)]++;
+    return plan_ar_batch(P) == SV_AR_COMP && n_eff > SV_MAX_TILE_FP32_REM &&
+           (states_of[n_eff] << (n_eff - SV_MAX_TILE_FP32_REM)) <= SV_FEW_STATES_TILES;
+  }
+  TileConfig task_tiles(uint32_t n_eff, bool fp64) {
+    TileConfig tc = tiles(n_eff, fp64);
+    if (!fp64 && !P->opts.tile_qubits && tc.k_max > SV_MAX_TILE_FP32_REM && few_states(n_eff)) {
+      tc.k_max = SV_MAX_TILE_FP32_REM;
+      if (!P->opts.low_qubits) tc.b = 3;
+    }
+    return tc;
+  }
+
   static double state_bytes(uint32_t mode, uint32_t n) {
     if (mode == QW_MODE_TABLEAU) return (double)(2 * n) * 2 * ((n + 63) / 64) * 8 + 2.0 * n;
     const uint32_t n_eff = std::max<uint32_t>(n, SV_G);
@@ -1045,7 +1068,7 @@ void build_plan(qw_plan *P, Engine *E, const Workload &W) {
                       ((tp.src >= 0) ? P->mats[tp.src].out_offset + P->mats[tp.src].tab_outs : 0);
     } else {
       T.copy_gates(tp.begin, T.n_gates, buf);
-      TileConfig tc = C.tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
+      TileConfig tc = C.task_tiles(tp.n_eff, T.mode == QW_MODE_SV_FP64);
       if (!P->opts.tile_qubits && sv_permutes(buf.data(), buf.size()))
         tc.k_max = sv_permute_tile(tp.n_eff, T.mode == QW_MODE_SV_FP64, tc.k_max);
       tp.sv = fuse_sv(buf.data(), buf.size(), tp.n_eff, tc, T.mode == QW_MODE_SV_FP64);

@@ -108,6 +108,9 @@ constexpr int SV_MAX_TILE_FP32_COMP = 13;
 // three CTAs per SM, 2^13 one (200 random gates at 24 qubits: 2.83 against
 // 3.58 ms)
 constexpr int SV_MAX_TILE_FP32_REM = 12;
+// compensated FP32 tasks of one size that are few enough for tiles of 2^12
+// amplitudes in place of the tuned ones: tiles of all their states together
+constexpr uint64_t SV_FEW_STATES_TILES = 1024;
 // a compensated FP32 task whose program has more passes than this keeps its
 // remainder between passes (rounding at every stage suits short suffixes
 // only; 40 mixed random-circuit tasks took 8.9 ms with a limit of 8 passes,
