@@ -1,5 +1,6 @@
 """Plans with few compensated states take tiles of 2^12 amplitudes where the
-tuner, which times many states, prefers wider ones.  Results against the oracle on both sides of the rule."""
+tuner, which times many states, prefers wider ones; where one of them keeps
+its remainder all do.  Results against the oracle on both sides of the rule."""
 import numpy as np
 import pytest
 
@@ -50,4 +51,12 @@ def test_tiles_follow_the_number_of_states(eng, count, tile):
     plan = Q.Plan(eng, Q.Workload(tasks), reuse=0).run()
     assert plan.cost_record()["wave_tiles"][0][0] == tile
     _check(plan, tasks, 16)
+    plan.close()
+
+
+def test_one_wave_for_chains_and_others(eng):
+    tasks = _tasks(16, 4, [40, 500, 60, 450])
+    plan = Q.Plan(eng, Q.Workload(tasks), reuse=0).run()
+    assert len(plan.cost_record()["wave_tiles"]) == 1
+    _check(plan, tasks, 1)
     plan.close()
