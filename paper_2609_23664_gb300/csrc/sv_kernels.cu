@@ -664,7 +664,10 @@ constexpr uint64_t WAIT_LIMIT_NS = 2000000000ull;  // 2 s per dependency wait
 // SV_AR_COMP) hold two FP32 complex values per amplitude in registers, 16
 // amplitudes per stage group, and are budgeted for three CTAs.
 // EN: the work list may hold energy blocks (option fuse_energy); their code
-// stays out of the ordinary build, whose registers it would spill.
+// stays out of the ordinary compensated build, whose registers it would
+// spill.  Plain FP32 has one build, with them: without, the compiler's
+// schedule of the stages is slower (400 gates at 6 qubits 141 us against 116,
+// 8 plain 22-qubit states 2016 against 1904).
 template <typename T, int MINB, int AR, int NT, bool EN>
 __global__ void __launch_bounds__(NT, MINB)
 sv_batch_kernel(SvTables t, const SvJob *__restrict__ jobs, const SvSeg *__restrict__ segs,
@@ -761,7 +764,8 @@ size_t sv_smem_bytes(bool fp64, uint32_t k, int ar) {
 }
 
 // the batch kernel of a precision, arithmetic and tile width: plain FP32 has
-// a 128-register build (four CTAs per SM) for tiles of at most 12 qubits
+// a 128-register build (four CTAs per SM) for tiles of at most 12 qubits, and
+// both with energy blocks
 typedef void (*SvBatchKernel)(SvTables, const SvJob *, const SvSeg *, uint32_t, uint32_t, unsigned int *, EnTables);
 template <bool EN>
 static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar, bool few = false) {
@@ -771,8 +775,8 @@ static SvBatchKernel batch_kernel_of(bool fp64, uint32_t k, int ar, bool few = f
     return few ? sv_batch_kernel<float, 1, SV_AR_REM, 256, false> : sv_batch_kernel<float, 3, SV_AR_REM, 128, false>;
   if constexpr (SV_G_PLAIN32 == 4) return sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, false>;
   else
-    return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, EN>
-                  : sv_batch_kernel<float, 4, SV_AR_PLAIN, SV_NT_PLAIN32, EN>;
+    return k > 12 ? sv_batch_kernel<float, 3, SV_AR_PLAIN, SV_NT_PLAIN32, true>
+                  : sv_batch_kernel<float, 4, SV_AR_PLAIN, SV_NT_PLAIN32, true>;
 }
 
 // Kernel attributes are set once, before any stream capture (a capture
@@ -790,8 +794,6 @@ cudaError_t sv_init_attrs() {
                      (const void *)batch_kernel_of<false>(true, 13, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<false>(false, 12, SV_AR_REM),
                      (const void *)batch_kernel_of<false>(false, 12, SV_AR_REM, true),
-                     (const void *)batch_kernel_of<true>(false, 13, SV_AR_PLAIN),
-                     (const void *)batch_kernel_of<true>(false, 12, SV_AR_PLAIN),
                      (const void *)batch_kernel_of<true>(false, 13, SV_AR_COMP),
                      (const void *)batch_kernel_of<true>(true, 13, SV_AR_PLAIN)};
   for (const void *f : k) {
