@@ -601,7 +601,8 @@ static void prepare(qw_plan *P) {
   D->task_pass0.assign(nt, 0);
   D->ar_batch = plan_ar_batch(P);
   D->ar_chain = D->ar_batch == SV_AR_COMP ? SV_AR_REM : SV_AR_PLAIN;
-  size_t rem_bytes = 0;  // largest FP32 chain that keeps a remainder
+  size_t rem_bytes = 0;      // largest FP32 chain launched pass by pass that keeps a remainder
+  size_t mat_rem_bytes = 0;  // and boundary
   for (size_t m = 0; m < P->mats.size(); m++) {
     const MatNode &M = P->mats[m];
     if (M.mode == QW_MODE_TABLEAU) continue;
@@ -612,7 +613,7 @@ static void prepare(qw_plan *P) {
     // algorithmic bytes of the boundary's passes (state, and the remainder between passes)
     P->prefix_alg_bytes += chain_bytes((double)S, M.sv.passes.size(), ar);
     for (const HostPass &hp : M.sv.passes) P->prefix_alg_flops += pass_flops(hp, M.n_eff, M.sv.g, ar);
-    if (ar == SV_AR_REM && M.sv.passes.size() > 1) rem_bytes = std::max(rem_bytes, S);
+    if (ar == SV_AR_REM && M.sv.passes.size() > 1) mat_rem_bytes = std::max(mat_rem_bytes, S);
   }
   for (uint32_t t = 0; t < nt; t++) {
     const TaskPlan &tp = P->tasks[t];
@@ -728,9 +729,9 @@ static void prepare(qw_plan *P) {
   // statevector boundary of its own precision (no export or conversion in
   // between); a boundary's first pass then waits for its parent's last, and
   // sibling boundaries run side by side.  Otherwise: pass by pass.
+  uint64_t mat_rem = 0;  // remainder arrays of every boundary
   {
     bool ok = P->opts.batched != 0;
-    uint64_t mat_rem = 0;  // remainder arrays of every boundary
     size_t n_sv = 0;
     for (const qw_dense_prog *dp : D->mat_dense)
       if (dp) ok = false;  // a dense-block boundary is launched block by block
@@ -748,7 +749,11 @@ static void prepare(qw_plan *P) {
     if (mat_rem > std::min<uint64_t>(MAT_REM_BYTES, E->task_budget / 8)) ok = false;
     // a single boundary is a chain of dependent passes: separate launches
     // serve it as well, without CTAs waiting on the previous pass
-    if (ok && n_sv > 1) {
+    ok = ok && n_sv > 1;
+    if (!ok) {
+      mat_rem = 0;
+      rem_bytes = mat_rem_bytes;
+    } else {
       std::vector<uint32_t> level(P->mats.size(), 0);
       uint32_t max_level = 0;
       size_t max_p = 0;
@@ -881,7 +886,7 @@ static void prepare(qw_plan *P) {
     std::map<std::pair<int, uint32_t>, bool> n_share;
     std::vector<std::pair<size_t, std::pair<int, uint32_t>>> order;  // (S, group)
     std::map<std::pair<int, uint32_t>, size_t> n_pooled;
-    uint64_t committed = 0;
+    uint64_t committed = mat_rem;  // the boundaries' remainder arrays come out of it too
     for (auto &g : groups) {
       size_t np = 0, nl = 0;
       bool pooled_long = false;
