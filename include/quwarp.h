@@ -143,7 +143,10 @@ typedef struct qw_engine_opts {
 } qw_engine_opts;
 
 /* Creates an engine on `opts->device` (NULL opts = defaults on device 0).
- * Owns the device memory it allocates and its internal streams.  Destroying
+ * Owns the device memory it allocates and its internal streams; up to 1 GB of
+ * workspace of the calls on caller buffers (qw_sv_*_dev) stays mapped between
+ * calls and is given back when a plan runs out of memory and with the engine.
+ * Destroying
  * an engine also releases the device memory of the plans created on it;
  * those plans keep their host results and EXPLAIN trace, but qw_execute and
  * qw_get_state on them return QW_ERR_STATE. */
@@ -473,8 +476,8 @@ qw_status qw_sv_sample_dev(qw_engine *e, uint32_t mode, uint32_t n, const void *
  * has reserved the pool), and latency-bound loops with a fixed memory
  * footprint that cannot pay the device synchronization of cudaFree.  It
  * computes what qw_sv_energy_dev computes, with the same kernels, but needs
- * no engine and allocates nothing: the term layout, the job record and the
- * per-block partial sums live in one fixed device array of the library
+ * no engine and allocates no device memory (the term layout is built on the host
+ * heap): layout, job record and per-block partial sums live in one fixed device array of the library
  * (about 1.1 MB, held by every GPU that loads the library until the process
  * exits).  Its term layout is bounded (at most 8 classes of terms), so above
  * 25 FP32 qubits its sums run in another order than qw_sv_energy_dev's.

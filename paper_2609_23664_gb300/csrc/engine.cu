@@ -917,8 +917,10 @@ static void prepare(qw_plan *P) {
   // where its tiles take at most half of the resident CTAs (up to 19 qubits:
   // 64 tiles of 18 qubits left 86 % idle), or where they take two or three
   // rounds of them and the last is less than half full (21 and 22 qubits: 512
-  // and 1024 tiles on 456 CTAs).  Other registers fill the chip alone and run
-  // one task after another, pass by pass.
+  // and 1024 tiles on 456 CTAs).  Other registers run one task after another,
+  // pass by pass.  From 23 qubits on they fill the chip alone; 20 qubits (256
+  // tiles) would leave 44 % of it idle, but sharing there makes a rerun of two
+  // tasks cheaper than Eq. 2, which prices passes of one state, estimates it.
   auto long_chain = [&](const TaskPlan &tp) { return batched && tp.chain; };
   const uint32_t rem_slots = (uint32_t)sv_batch_grid(false, SV_MAX_TILE_FP32_REM, E->sm_count, SV_AR_REM);
   auto shares_launch = [&](const TaskPlan &tp) {
