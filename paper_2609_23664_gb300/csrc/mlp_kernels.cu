@@ -137,22 +137,34 @@ mlp_kernel(const float *__restrict__ P, const float *__restrict__ X, const float
 }
 
 // grad[p] = sum over CTAs of partial[c][p], loss likewise / batch: slices of
-// the CTAs in order, then the slices in order
+// the CTAs in order, then the slices in order.  The sums are kept in pairs
+// (two-sum): with a partial per three samples instead of 32, plain ones erred by
+// more than those had (median over batches of 256: 8.2e-8 of the gradient's
+// norm, 7.0e-8 with CTAs of 32, 4.0e-8 in pairs)
 constexpr int RED_P = 32, RED_S = 16;  // parameters and slices per CTA
 __global__ void __launch_bounds__(RED_P * RED_S)
 mlp_reduce_kernel(const float *__restrict__ partial, uint32_t n_cta, uint32_t batch, float *grad, float *loss) {
-  __shared__ float red[RED_S][RED_P];
+  __shared__ float2 red[RED_S][RED_P];
   const uint32_t l = threadIdx.x % RED_P, z = threadIdx.x / RED_P, p = blockIdx.x * RED_P + l;
   const uint32_t per = (n_cta + RED_S - 1) / RED_S, c1 = min(n_cta, (z + 1) * per);
-  float s = 0.f;
+  float hi = 0.f, lo = 0.f;
+  auto add = [&](float v) {
+    const float t = hi + v, b = t - hi;
+    lo += (hi - (t - b)) + (v - b);
+    hi = t;
+  };
   if (p <= (uint32_t)N_PARAMS) {
 #pragma unroll 8
-    for (uint32_t c = z * per; c < c1; c++) s += partial[(size_t)c * (N_PARAMS + 1) + p];
+    for (uint32_t c = z * per; c < c1; c++) add(partial[(size_t)c * (N_PARAMS + 1) + p]);
   }
-  red[z][l] = s;
+  red[z][l] = make_float2(hi, lo);
   __syncthreads();
   if (z != 0 || p > (uint32_t)N_PARAMS) return;
-  for (int k = 1; k < RED_S; k++) s += red[k][l];
+  for (int k = 1; k < RED_S; k++) {
+    add(red[k][l].x);
+    lo += red[k][l].y;
+  }
+  const float s = fabsf(hi) <= 3.402823466e38f ? hi + lo : hi;  // (an infinite sum has no low part)
   if (p < (uint32_t)N_PARAMS) grad[p] = s;
   else if (loss) *loss = s / (float)batch;
 }
